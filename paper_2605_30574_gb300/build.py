@@ -2,6 +2,7 @@
 
 * ``libsplice.so``        -- the spliced decode-attention library (C ABI in
   ``include/splice.h``), from ``csrc/``.
+* ``decoder/libsplice_decoder.so`` -- the decoder's elementwise kernels.
 * ``synth/libsplice_synth.so`` -- the device twin of the seeded input generator.
 
 Each translation unit is compiled by its own ``nvcc`` process, in parallel,
@@ -74,20 +75,27 @@ def synth_lib_path() -> str:
     return os.path.join(PKG, "synth", "libsplice_synth.so")
 
 
+def decoder_lib_path() -> str:
+    return os.path.join(PKG, "decoder", "libsplice_decoder.so")
+
+
 def build(force: bool = False, verbose: bool = False) -> None:
     csrc = os.path.join(PKG, "csrc")
     sources = sorted(glob.glob(os.path.join(csrc, "*.cu")) + glob.glob(os.path.join(csrc, "*.cpp")))
     headers = sorted(glob.glob(os.path.join(csrc, "*.h")) + glob.glob(os.path.join(csrc, "*.cuh")) +
                      glob.glob(os.path.join(ROOT, "include", "*.h")))
     synth_src = [os.path.join(PKG, "synth", "synth.cu")]
-    with cf.ThreadPoolExecutor(max_workers=2) as ex:
+    decoder_src = [os.path.join(PKG, "decoder", "decoder.cu")]
+    with cf.ThreadPoolExecutor(max_workers=3) as ex:
         a = ex.submit(build_lib, "splice", sources, headers, splice_lib_path(), force, verbose)
         b = ex.submit(build_lib, "synth", synth_src, [], synth_lib_path(), force, verbose)
+        c = ex.submit(build_lib, "decoder", decoder_src, [], decoder_lib_path(), force, verbose)
         a.result()
         b.result()
+        c.result()
 
 
 if __name__ == "__main__":
     import sys
     build(force="--force" in sys.argv, verbose=True)
-    print("built", splice_lib_path(), synth_lib_path())
+    print("built", splice_lib_path(), decoder_lib_path(), synth_lib_path())

@@ -1,0 +1,146 @@
+"""ctypes binding of the decoder's elementwise kernels (``libsplice_decoder.so``).
+
+``model.py`` calls these in place of the torch expressions next to them
+whenever nothing but the values is asked for (``plain``): eager CUDA tensors
+of the decoder's own types, with no gradient, transform, mode or autocast that
+would have to see the single operations.  Every launch goes to torch's current
+stream, and every output is allocated here.
+"""
+from __future__ import annotations
+
+import ctypes
+import os
+
+import torch
+import torch.autograd.forward_ad as _fwad
+
+_LIB = None
+POSITIONS = {torch.int64: 0, torch.int32: 1, torch.float32: 2}
+BF16, F32 = torch.bfloat16, torch.float32
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda device: torch.cuda.current_stream(device).cuda_stream)
+_current_device = torch.cuda.current_device
+
+
+def lib() -> ctypes.CDLL:
+    global _LIB
+    if _LIB is None:
+        path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libsplice_decoder.so")
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is not built: run paper_2605_30574_gb300.build.build()")
+        L = ctypes.CDLL(path)
+        vp, i, l, f = ctypes.c_void_p, ctypes.c_int, ctypes.c_long, ctypes.c_float
+        L.decoder_rms_norm.argtypes = [vp, vp, vp, l, i, f, vp]
+        L.decoder_add_rms_norm.argtypes = [vp, vp, vp, vp, vp, l, i, f, vp]
+        L.decoder_add.argtypes = [vp, vp, vp, l, vp]
+        L.decoder_to_bf16.argtypes = [vp, vp, l, vp]
+        L.decoder_silu_mul.argtypes = [vp, vp, l, vp, l, i, vp]
+        L.decoder_qkv_post.argtypes = [vp, vp, vp, vp, vp, vp, ctypes.POINTER(l), vp, vp, vp, vp, i, l, i, i, i, f, vp]
+        for fn in (L.decoder_rms_norm, L.decoder_add_rms_norm, L.decoder_add, L.decoder_to_bf16, L.decoder_silu_mul,
+                   L.decoder_qkv_post):
+            fn.restype = i
+        _LIB = L
+    return _LIB
+
+
+def plain(acts, weights) -> bool:
+    """Whether the kernels may stand in for the torch expressions on these
+    activations and bf16 weights."""
+    dev = acts[0].device
+    if dev.type != "cuda" or dev.index != torch.cuda.current_device():
+        return False
+    if (torch._C._are_functorch_transforms_active() or torch._C._len_torch_dispatch_stack()
+            or torch._C._len_torch_function_stack() or torch.is_autocast_enabled() or _fwad._current_level >= 0
+            or torch.compiler.is_compiling() or torch.jit.is_tracing()):
+        return False
+    grad = torch.is_grad_enabled()
+    for t in acts:
+        if type(t) is not torch.Tensor or t.device != dev or not t.is_contiguous() or (grad and t.requires_grad) \
+                or t.numel() == 0:
+            return False
+    for t in weights:
+        if t.dtype is not BF16 or t.device != dev or not t.is_contiguous() or (grad and t.requires_grad) \
+                or type(t) not in (torch.Tensor, torch.nn.Parameter):
+            return False
+    return True
+
+
+def joined(*ws):
+    """The matrices as one, when they are consecutive rows of one contiguous
+    matrix (as the decoder lays them out), else None."""
+    base = ws[0]._base
+    if base is None or base.dim() != 2 or not base.is_contiguous() or base.dtype is not ws[0].dtype:
+        return None
+    at = base.data_ptr()
+    for w in ws:
+        if w._base is not base or w.data_ptr() != at or w.shape[1] != base.shape[1]:
+            return None
+        at += w.numel() * w.element_size()
+    return base if sum(w.shape[0] for w in ws) == base.shape[0] else None
+
+
+def _launch(name, *args):
+    # (the raw handle of torch's current stream: a Stream object costs more
+    # host time than the launch)
+    rc = getattr(_LIB or lib(), name)(*args, _raw_stream(_current_device()))
+    if rc != 0:
+        raise RuntimeError(f"{name} failed with CUDA error {rc}")
+
+
+def _rows(t):
+    return t.numel() // t.shape[-1]
+
+
+def _like(t, dtype):
+    return torch.empty(t.shape, dtype=dtype, device=t.device)
+
+
+def rms_norm(h, w, eps):
+    """bf16(h / rms(h) * w) of fp32 rows."""
+    x = _like(h, BF16)
+    _launch("decoder_rms_norm", h.data_ptr(), w.data_ptr(), x.data_ptr(), _rows(h), h.shape[-1], eps)
+    return x
+
+
+def add_rms_norm(h, o, w, eps):
+    """h + o and the bf16 norm of the sum."""
+    h2, x = _like(h, F32), _like(h, BF16)
+    _launch("decoder_add_rms_norm", h.data_ptr(), o.data_ptr(), w.data_ptr(), h2.data_ptr(), x.data_ptr(), _rows(h),
+            h.shape[-1], eps)
+    return h2, x
+
+
+def add_(h, o):
+    """h += o (o bf16)."""
+    _launch("decoder_add", h.data_ptr(), o.data_ptr(), h.data_ptr(), h.numel())
+    return h
+
+
+def to_bf16(x):
+    y = _like(x, BF16)
+    _launch("decoder_to_bf16", x.data_ptr(), y.data_ptr(), x.numel())
+    return y
+
+
+def silu_mul(gate, up):
+    """bf16(silu(gate) * up)."""
+    f, y = gate.shape[-1], _like(gate, BF16)
+    _launch("decoder_silu_mul", gate.data_ptr(), up.data_ptr(), f, y.data_ptr(), _rows(gate), f)
+    return y
+
+
+def silu_mul_joined(gate_up):
+    """The same for rows that hold gate, then up."""
+    f = gate_up.shape[-1] // 2
+    y = torch.empty((*gate_up.shape[:-1], f), dtype=BF16, device=gate_up.device)
+    p = gate_up.data_ptr()
+    _launch("decoder_silu_mul", p, p + 2 * f, 2 * f, y.data_ptr(), _rows(y), f)
+    return y
+
+
+def qkv_post(q, k, v, strides, outs, out_strides, q_norm, k_norm, inv_freq, pos, hq, hkv, d, eps):
+    """Per-head norm and RoPE of q and k, and v as it is.  q, k, v: pointers of
+    the projections' rows, ``strides`` elements apart; outs: the three output
+    pointers, with (row, head) strides each."""
+    _launch("decoder_qkv_post", q, k, v, *outs, (ctypes.c_long * 9)(*strides, *out_strides), q_norm.data_ptr(),
+            k_norm.data_ptr(), inv_freq.data_ptr(), pos.data_ptr(), POSITIONS[pos.dtype], pos.numel(), hq, hkv, d, eps)

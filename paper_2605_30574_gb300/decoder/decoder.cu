@@ -1,0 +1,368 @@
+// Elementwise and normalisation kernels of the decoder that drives Algorithm 1
+// (model.py): RMSNorm, the per-head norm and RoPE of q and k, the residual
+// additions, SwiGLU's product and the attention output's conversion.  The
+// projections between them are library GEMMs, the decode attention is
+// libsplice.so's.
+//
+// Every kernel reads its inputs once and writes its outputs once, computes in
+// fp32 and rounds to bf16 only where the decoder's definition does (model.py's
+// torch expressions: the norm's output, q and k after RoPE, the SwiGLU product,
+// the attention output), with the same order of the element operations; only
+// the order of the row sums differs.
+//
+// At a decode batch each of them moves 10-50 MB: one wave or a few of blocks
+// that are bound by their loads' latency, not by bandwidth.  Their point is
+// their number: in a Qwen3-8B-shaped layer of 512 cells they take the place
+// of 62 launches by 7 (980 -> 317 us; a step of two layers and the head 2149
+// -> 797, a prefill of 1024 tokens 2376 -> 890).  Times below are a launch's
+// on cold caches at 512 rows of 4096 (32 + 2 x 8 heads of 128, F = 12288).
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kKeep = 4;        // float4 of a row that a thread keeps in registers between the passes
+
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    return x;
+}
+
+__device__ __forceinline__ uint2 pack4(float a, float b, float c, float d) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+}
+
+__device__ __forceinline__ float4 unpack4(uint2 w) {
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                       __uint_as_float(w.y & 0xffff0000u));
+}
+
+__device__ __forceinline__ float4 add4(float4 a, float4 b) {
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+// x = bf16(h / rms(h) * w), one block per row; ADD: h + o first (o bf16, the
+// output of a projection), the sum written to h2.  6 bytes per element (ADD:
+// 12): 6.9 us, ADD 5.8 (the five torch passes it replaces: 33).  A thread keeps its first kKeep float4 of the row in
+// registers, so rows of up to 4096 elements are read once; what is beyond is
+// read again for the second pass (from L1 or L2).
+template <bool ADD, bool VEC>
+__global__ void __launch_bounds__(kThreads)
+    rms_norm_kernel(const float* __restrict__ h, const __nv_bfloat16* __restrict__ o,
+                    const __nv_bfloat16* __restrict__ w, float* __restrict__ h2, __nv_bfloat16* __restrict__ x, int D,
+                    float eps) {
+    __shared__ float part[kThreads / 32];
+    const size_t base = size_t(blockIdx.x) * D;
+    const int t = threadIdx.x;
+    float sum = 0.f;
+    float4 keep[kKeep];
+    const int n4 = VEC ? D / 4 : 0;
+    auto load4 = [&](int i) -> float4 {
+        float4 v = reinterpret_cast<const float4*>(h + base)[i];
+        if (ADD) v = add4(v, unpack4(reinterpret_cast<const uint2*>(o + base)[i]));
+        return v;
+    };
+    auto load1 = [&](int i) -> float { return ADD ? h[base + i] + __bfloat162float(o[base + i]) : h[base + i]; };
+    if constexpr (VEC) {
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            const int i = t + k * kThreads;
+            keep[k] = i < n4 ? load4(i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            const int i = t + k * kThreads;
+            if (ADD && i < n4) reinterpret_cast<float4*>(h2 + base)[i] = keep[k];
+            sum += (keep[k].x * keep[k].x + keep[k].y * keep[k].y) + (keep[k].z * keep[k].z + keep[k].w * keep[k].w);
+        }
+        for (int i = t + kKeep * kThreads; i < n4; i += kThreads) {
+            const float4 v = load4(i);
+            if (ADD) reinterpret_cast<float4*>(h2 + base)[i] = v;
+            sum += (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
+        }
+    } else {
+        for (int i = t; i < D; i += kThreads) {
+            const float v = load1(i);
+            if (ADD) h2[base + i] = v;
+            sum += v * v;
+        }
+    }
+    sum = warp_sum(sum);
+    if ((t & 31) == 0) part[t >> 5] = sum;
+    __syncthreads();
+    sum = 0.f;
+#pragma unroll
+    for (int k = 0; k < kThreads / 32; ++k) sum += part[k];
+    const float r = rsqrtf(sum / float(D) + eps);
+    if constexpr (VEC) {
+        auto out4 = [&](int i, float4 v) {
+            const float4 g = unpack4(reinterpret_cast<const uint2*>(w)[i]);
+            reinterpret_cast<uint2*>(x + base)[i] =
+                pack4(__fmul_rn(v.x * r, g.x), __fmul_rn(v.y * r, g.y), __fmul_rn(v.z * r, g.z), __fmul_rn(v.w * r, g.w));
+        };
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k) {
+            const int i = t + k * kThreads;
+            if (i < n4) out4(i, keep[k]);
+        }
+        for (int i = t + kKeep * kThreads; i < n4; i += kThreads) out4(i, load4(i));
+    } else {
+        for (int i = t; i < D; i += kThreads)
+            x[base + i] = __float2bfloat16_rn(__fmul_rn(load1(i) * r, __bfloat162float(w[i])));
+    }
+}
+
+// h2 = h + o (o bf16); h2 may be h.  10 bytes per element: 5.0 us.
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads)
+    add_kernel(const float* h, const __nv_bfloat16* __restrict__ o, float* h2, long n) {
+    const long i = long(blockIdx.x) * kThreads + threadIdx.x;
+    if constexpr (VEC) {
+        if (i < n / 4)
+            reinterpret_cast<float4*>(h2)[i] =
+                add4(reinterpret_cast<const float4*>(h)[i], unpack4(reinterpret_cast<const uint2*>(o)[i]));
+    } else {
+        if (i < n) h2[i] = h[i] + __bfloat162float(o[i]);
+    }
+}
+
+// y = bf16(x): 6 bytes per element, 4.2 us.
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads)
+    to_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ y, long n) {
+    const long i = long(blockIdx.x) * kThreads + threadIdx.x;
+    if constexpr (VEC) {
+        if (i < n / 4) {
+            const float4 v = reinterpret_cast<const float4*>(x)[i];
+            reinterpret_cast<uint2*>(y)[i] = pack4(v.x, v.y, v.z, v.w);
+        }
+    } else {
+        if (i < n) y[i] = __float2bfloat16_rn(x[i]);
+    }
+}
+
+__device__ __forceinline__ float silu(float g) { return g / (1.f + expf(-g)); }
+
+// y[r][i] = bf16(silu(gate[r][i]) * up[r][i]); gate and up rows are `ld`
+// elements apart (2 F when one GEMM made both).  6 bytes per output: 9.9 us
+// (38 MB, 3.8 TB/s).
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads)
+    silu_mul_kernel(const __nv_bfloat16* __restrict__ gate, const __nv_bfloat16* __restrict__ up, long ld,
+                    __nv_bfloat16* __restrict__ y, int F) {
+    const long r = blockIdx.y;
+    const int i = blockIdx.x * kThreads + threadIdx.x;
+    if constexpr (VEC) {
+        if (i >= F / 4) return;
+        const float4 g = unpack4(reinterpret_cast<const uint2*>(gate + r * ld)[i]);
+        const float4 u = unpack4(reinterpret_cast<const uint2*>(up + r * ld)[i]);
+        reinterpret_cast<uint2*>(y + r * F)[i] = pack4(silu(g.x) * u.x, silu(g.y) * u.y, silu(g.z) * u.z, silu(g.w) * u.w);
+    } else {
+        if (i >= F) return;
+        y[r * F + i] = __float2bfloat16_rn(silu(__bfloat162float(gate[r * ld + i])) * __bfloat162float(up[r * ld + i]));
+    }
+}
+
+struct HeadRows {
+    const __nv_bfloat16* src;   // rows [row][head][d], rows `ld` elements apart
+    long ld;
+    __nv_bfloat16* dst;         // element (row, head, c) at row * row_stride + head * head_stride + c
+    long row_stride, head_stride;
+};
+
+// V bf16 values, loaded and stored as one word.
+template <int V>
+struct alignas(2 * V) Vec {
+    __nv_bfloat16 x[V];
+};
+
+// q and k: bf16(rope(rms_norm over the head dim)); v: copied.  A warp per
+// (row, head), eight heads of a row per block; the row's D / 2 rotation
+// angles are computed once per block into shared memory.  Lane i holds
+// elements V i .. V i + V - 1 of both halves of the head (V = D / 64), so the
+// rotation needs no exchange.  4 bytes per element and one head per warp, so
+// that a row's 48 heads are in flight at once: 8.0 us, where torch made 36
+// launches.  Pointers are 16-byte aligned and strides
+// multiples of 8 (the caller checks).
+template <int D>
+__global__ void __launch_bounds__(kThreads)
+    qkv_post_kernel(HeadRows q, HeadRows k, HeadRows v, const __nv_bfloat16* __restrict__ q_norm,
+                    const __nv_bfloat16* __restrict__ k_norm, const float* __restrict__ inv_freq,
+                    const void* __restrict__ pos, int pos_kind, int Hq, int Hkv, float eps) {
+    constexpr int HALF = D / 2, V = D / 64;
+    __shared__ float2 cs[HALF];
+    const long row = blockIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int j = blockIdx.y * (kThreads / 32) + warp;
+    const bool live = j < Hq + 2 * Hkv, turn = j < Hq + Hkv;
+    const __nv_bfloat16* src = nullptr;
+    __nv_bfloat16* dst = nullptr;
+    if (j < Hq) {
+        src = q.src + row * q.ld + long(j) * D;
+        dst = q.dst + row * q.row_stride + j * q.head_stride;
+    } else if (turn) {
+        src = k.src + row * k.ld + long(j - Hq) * D;
+        dst = k.dst + row * k.row_stride + (j - Hq) * k.head_stride;
+    } else if (live) {
+        src = v.src + row * v.ld + long(j - Hq - Hkv) * D;
+        dst = v.dst + row * v.row_stride + (j - Hq - Hkv) * v.head_stride;
+    }
+    Vec<V> lo, hi, g_lo, g_hi;
+    if (live) {
+        lo = reinterpret_cast<const Vec<V>*>(src)[lane];
+        hi = reinterpret_cast<const Vec<V>*>(src + HALF)[lane];
+    }
+    if (turn) {
+        const __nv_bfloat16* g = j < Hq ? q_norm : k_norm;
+        g_lo = reinterpret_cast<const Vec<V>*>(g)[lane];
+        g_hi = reinterpret_cast<const Vec<V>*>(g + HALF)[lane];
+    }
+    float p;
+    if (pos_kind == 0)
+        p = float(reinterpret_cast<const int64_t*>(pos)[row]);
+    else if (pos_kind == 1)
+        p = float(reinterpret_cast<const int32_t*>(pos)[row]);
+    else
+        p = reinterpret_cast<const float*>(pos)[row];
+    for (int i = threadIdx.x; i < HALF; i += kThreads) {
+        float s, c;
+        sincosf(p * inv_freq[i], &s, &c);
+        cs[i] = make_float2(c, s);
+    }
+    __syncthreads();
+    if (!live) return;
+    if (turn) {
+        float a[V], b[V], sum = 0.f;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            a[i] = __bfloat162float(lo.x[i]);
+            b[i] = __bfloat162float(hi.x[i]);
+            sum += a[i] * a[i] + b[i] * b[i];
+        }
+        const float r = rsqrtf(warp_sum(sum) / float(D) + eps);
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            const float x1 = __fmul_rn(a[i] * r, __bfloat162float(g_lo.x[i]));
+            const float x2 = __fmul_rn(b[i] * r, __bfloat162float(g_hi.x[i]));
+            const float2 f = cs[lane * V + i];
+            lo.x[i] = __float2bfloat16_rn(__fsub_rn(__fmul_rn(x1, f.x), __fmul_rn(x2, f.y)));
+            hi.x[i] = __float2bfloat16_rn(__fadd_rn(__fmul_rn(x2, f.x), __fmul_rn(x1, f.y)));
+        }
+    }
+    reinterpret_cast<Vec<V>*>(dst)[lane] = lo;
+    reinterpret_cast<Vec<V>*>(dst + HALF)[lane] = hi;
+}
+
+bool vec_ok(const void* a, const void* b, const void* c, const void* d, long n) {
+    const uintptr_t bits = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) |
+                           reinterpret_cast<uintptr_t>(c) | reinterpret_cast<uintptr_t>(d);
+    return (bits & 15u) == 0 && n % 4 == 0;
+}
+
+unsigned blocks_for(long n) { return unsigned((n + kThreads - 1) / kThreads); }
+
+using bf = __nv_bfloat16;
+
+}  // namespace
+
+// Every call returns the cudaError_t of its launch and takes contiguous rows
+// unless strides are given; rows and sizes >= 1.  rows < 2^31, n < 2^39.
+extern "C" {
+
+int decoder_rms_norm(const void* h, const void* w, void* x, long rows, int D, float eps, void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (vec_ok(h, w, x, nullptr, D))
+        rms_norm_kernel<false, true><<<unsigned(rows), kThreads, 0, st>>>(
+            static_cast<const float*>(h), nullptr, static_cast<const bf*>(w), nullptr, static_cast<bf*>(x), D, eps);
+    else
+        rms_norm_kernel<false, false><<<unsigned(rows), kThreads, 0, st>>>(
+            static_cast<const float*>(h), nullptr, static_cast<const bf*>(w), nullptr, static_cast<bf*>(x), D, eps);
+    return int(cudaGetLastError());
+}
+
+int decoder_add_rms_norm(const void* h, const void* o, const void* w, void* h2, void* x, long rows, int D, float eps,
+                         void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (vec_ok(h, w, x, h2, D) && vec_ok(o, nullptr, nullptr, nullptr, D))
+        rms_norm_kernel<true, true><<<unsigned(rows), kThreads, 0, st>>>(
+            static_cast<const float*>(h), static_cast<const bf*>(o), static_cast<const bf*>(w),
+            static_cast<float*>(h2), static_cast<bf*>(x), D, eps);
+    else
+        rms_norm_kernel<true, false><<<unsigned(rows), kThreads, 0, st>>>(
+            static_cast<const float*>(h), static_cast<const bf*>(o), static_cast<const bf*>(w),
+            static_cast<float*>(h2), static_cast<bf*>(x), D, eps);
+    return int(cudaGetLastError());
+}
+
+int decoder_add(const void* h, const void* o, void* h2, long n, void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (vec_ok(h, o, h2, nullptr, n))
+        add_kernel<true><<<blocks_for(n / 4), kThreads, 0, st>>>(static_cast<const float*>(h),
+                                                                 static_cast<const bf*>(o), static_cast<float*>(h2), n);
+    else
+        add_kernel<false><<<blocks_for(n), kThreads, 0, st>>>(static_cast<const float*>(h), static_cast<const bf*>(o),
+                                                              static_cast<float*>(h2), n);
+    return int(cudaGetLastError());
+}
+
+int decoder_to_bf16(const void* x, void* y, long n, void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (vec_ok(x, y, nullptr, nullptr, n))
+        to_bf16_kernel<true><<<blocks_for(n / 4), kThreads, 0, st>>>(static_cast<const float*>(x),
+                                                                     static_cast<bf*>(y), n);
+    else
+        to_bf16_kernel<false><<<blocks_for(n), kThreads, 0, st>>>(static_cast<const float*>(x), static_cast<bf*>(y), n);
+    return int(cudaGetLastError());
+}
+
+int decoder_silu_mul(const void* gate, const void* up, long ld, void* y, long rows, int F, void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // (blockIdx.y holds a row: at most 65535 rows per launch)
+    for (long r0 = 0; r0 < rows; r0 += 65535) {
+        const unsigned n = unsigned(rows - r0 < 65535 ? rows - r0 : 65535);
+        const bf* g = static_cast<const bf*>(gate) + r0 * ld;
+        const bf* u = static_cast<const bf*>(up) + r0 * ld;
+        bf* out = static_cast<bf*>(y) + r0 * F;
+        if (vec_ok(g, u, out, nullptr, F) && ld % 8 == 0)
+            silu_mul_kernel<true><<<dim3(blocks_for(F / 4), n), kThreads, 0, st>>>(g, u, ld, out, F);
+        else
+            silu_mul_kernel<false><<<dim3(blocks_for(F), n), kThreads, 0, st>>>(g, u, ld, out, F);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return int(e);
+    }
+    return 0;
+}
+
+// strides: {q, k, v source row strides, q row, q head, k row, k head, v row, v
+// head destination strides}, in elements.  pos_kind: 0 int64, 1 int32, 2 fp32.
+int decoder_qkv_post(const void* q, const void* k, const void* v, void* q_out, void* k_out, void* v_out,
+                     const long* strides, const void* q_norm, const void* k_norm, const void* inv_freq,
+                     const void* pos, int pos_kind, long rows, int Hq, int Hkv, int d, float eps, void* stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const HeadRows a{static_cast<const bf*>(q), strides[0], static_cast<bf*>(q_out), strides[3], strides[4]};
+    const HeadRows b{static_cast<const bf*>(k), strides[1], static_cast<bf*>(k_out), strides[5], strides[6]};
+    const HeadRows c{static_cast<const bf*>(v), strides[2], static_cast<bf*>(v_out), strides[7], strides[8]};
+    const bf* qn = static_cast<const bf*>(q_norm);
+    const bf* kn = static_cast<const bf*>(k_norm);
+    const float* fr = static_cast<const float*>(inv_freq);
+    const dim3 grid(unsigned(rows), unsigned((Hq + 2 * Hkv + kThreads / 32 - 1) / (kThreads / 32)));
+    switch (d) {
+        case 64:
+            qkv_post_kernel<64><<<grid, kThreads, 0, st>>>(a, b, c, qn, kn, fr, pos, pos_kind, Hq, Hkv, eps);
+            break;
+        case 128:
+            qkv_post_kernel<128><<<grid, kThreads, 0, st>>>(a, b, c, qn, kn, fr, pos, pos_kind, Hq, Hkv, eps);
+            break;
+        case 256:
+            qkv_post_kernel<256><<<grid, kThreads, 0, st>>>(a, b, c, qn, kn, fr, pos, pos_kind, Hq, Hkv, eps);
+            break;
+        default: return int(cudaErrorInvalidValue);
+    }
+    return int(cudaGetLastError());
+}
+
+}  // extern "C"

@@ -35,6 +35,7 @@ from typing import List, Optional, Sequence
 
 import torch
 
+from . import decoder as K
 from . import splice as S
 from .synth import workloads as W
 
@@ -84,14 +85,24 @@ class RandomDecoder:
         def rnd(*shape, scale=std):
             return (torch.randn(*shape, generator=g, dtype=torch.float32, device=self.device) * scale).to(torch.bfloat16)
 
+        def rows(*heights):
+            # matrices that read the same input, as consecutive rows of one:
+            # one GEMM gives all their outputs
+            m = torch.cat([rnd(n, dims.d_model) for n in heights])
+            ends = [sum(heights[:i + 1]) for i in range(len(heights))]
+            return [m[e - n:e] for n, e in zip(heights, ends)]
+
         D, Hq, Hkv, d, F = dims.d_model, dims.num_q_heads, dims.num_kv_heads, dims.head_dim, dims.ffn
         self.embed = rnd(dims.vocab, D, scale=1.0)
         self.layers = []
         for _ in range(dims.num_layers):
+            wq, wk, wv = rows(Hq * d, Hkv * d, Hkv * d)
+            wo = rnd(D, Hq * d)
+            w_gate, w_up = rows(F, F)
             self.layers.append(dict(
-                in_norm=torch.ones(D, **bf), wq=rnd(Hq * d, D), wk=rnd(Hkv * d, D), wv=rnd(Hkv * d, D),
-                q_norm=torch.ones(d, **bf), k_norm=torch.ones(d, **bf), wo=rnd(D, Hq * d),
-                post_norm=torch.ones(D, **bf), w_gate=rnd(F, D), w_up=rnd(F, D), w_down=rnd(D, F)))
+                in_norm=torch.ones(D, **bf), wq=wq, wk=wk, wv=wv, q_norm=torch.ones(d, **bf),
+                k_norm=torch.ones(d, **bf), wo=wo, post_norm=torch.ones(D, **bf), w_gate=w_gate, w_up=w_up,
+                w_down=rnd(D, F)))
         self.final_norm = torch.ones(D, **bf)
         self.lm_head = rnd(dims.vocab, D)
         half = d // 2
@@ -110,6 +121,11 @@ class RandomDecoder:
     def qkv(self, l: int, h: torch.Tensor, pos: torch.Tensor):
         """h [..., n, D] fp32, pos [..., n] -> q [..., n, Hq, d], k, v [..., n, Hkv, d] (bf16)."""
         dims, w = self.dims, self.layers[l]
+        if self._kernels(l, h, pos):
+            q, k, v = (torch.empty((*h.shape[:-1], n, dims.head_dim), dtype=torch.bfloat16, device=h.device)
+                       for n in (dims.num_q_heads, dims.num_kv_heads, dims.num_kv_heads))
+            self._qkv_into(l, K.rms_norm(h, w["in_norm"], dims.rms_eps), pos, q, k, v)
+            return q, k, v
         x = _rms_norm(h, w["in_norm"], dims.rms_eps).to(torch.bfloat16)
         q = (x @ w["wq"].t()).unflatten(-1, (dims.num_q_heads, dims.head_dim))
         k = (x @ w["wk"].t()).unflatten(-1, (dims.num_kv_heads, dims.head_dim))
@@ -121,6 +137,9 @@ class RandomDecoder:
     def block_out(self, l: int, h: torch.Tensor, attn: torch.Tensor) -> torch.Tensor:
         """Residual stream after layer l given its attention output attn [..., Hq, d]."""
         dims, w = self.dims, self.layers[l]
+        if self._kernels(l, h) and self._attn_ok(h, attn):
+            h, o = self._block(l, h, attn)
+            return K.add_(h, o)
         h = h + (attn.to(torch.bfloat16).flatten(-2) @ w["wo"].t()).float()
         x = _rms_norm(h, w["post_norm"], dims.rms_eps).to(torch.bfloat16)
         gate = x @ w["w_gate"].t()
@@ -128,8 +147,82 @@ class RandomDecoder:
         return h + ((torch.nn.functional.silu(gate.float()) * up.float()).to(torch.bfloat16) @ w["w_down"].t()).float()
 
     def logits(self, h: torch.Tensor) -> torch.Tensor:
+        if (h.dtype is torch.float32 and h.shape[-1:] == self.final_norm.shape == self.lm_head.shape[1:]
+                and K.plain((h,), (self.final_norm, self.lm_head))):
+            x = K.rms_norm(h, self.final_norm, self.dims.rms_eps)
+            # (the product's fp32 sums as they are, in one pass over the logits)
+            return torch.mm(x.flatten(0, -2) if x.dim() > 1 else x[None], self.lm_head.t(),
+                            out_dtype=torch.float32).view(*h.shape[:-1], -1)
         x = _rms_norm(h, self.final_norm, self.dims.rms_eps).to(torch.bfloat16)
         return (x @ self.lm_head.t()).float()
+
+    # -- the same pieces through the library's kernels ----------------------
+    # The torch expressions above take about 70 launches per layer, and on
+    # this part's host the launches, not the kernels, set the time (a
+    # Qwen3-8B-shaped layer at batch 512: 1010 of 1087 us were host time).
+    # Here every run of elementwise operations is one kernel and matrices that
+    # read the same rows are one GEMM.
+    def _kernels(self, l: int, h: torch.Tensor, pos: Optional[torch.Tensor] = None) -> bool:
+        """Whether the kernels apply to these inputs and layer l's weights: its
+        projections and RoPE (pos given), or what follows its attention."""
+        dims, w = self.dims, self.layers[l]
+        D, d, nq, nk = dims.d_model, dims.head_dim, dims.num_q_heads * dims.head_dim, dims.num_kv_heads * dims.head_dim
+        if h.dtype is not torch.float32 or h.shape[-1:] != (D,):
+            return False
+        if pos is None:
+            return (w["wo"].shape == (D, nq) and w["post_norm"].shape == (D,)
+                    and w["w_gate"].shape == w["w_up"].shape == w["w_down"].shape[::-1]
+                    and K.plain((h,), (w["wo"], w["post_norm"], w["w_gate"], w["w_up"], w["w_down"])))
+        return (d in (64, 128, 256) and h.dim() >= 2 and pos.dtype in K.POSITIONS and pos.shape == h.shape[:-1]
+                and self.inv_freq.dtype is torch.float32 and self.inv_freq.shape == (d // 2,)
+                and w["in_norm"].shape == (D,) and w["q_norm"].shape == w["k_norm"].shape == (d,)
+                and w["wq"].shape == (nq, D) and w["wk"].shape == w["wv"].shape == (nk, D)
+                and K.plain((h, pos, self.inv_freq),
+                            (w["in_norm"], w["wq"], w["wk"], w["wv"], w["q_norm"], w["k_norm"])))
+
+    def _attn_ok(self, h: torch.Tensor, attn: torch.Tensor) -> bool:
+        """Whether the attention output is laid out as the kernels read it."""
+        dims = self.dims
+        return (attn.dtype in (torch.float32, torch.bfloat16)
+                and attn.shape == (*h.shape[:-1], dims.num_q_heads, dims.head_dim) and K.plain((attn,), ()))
+
+    def _store_ok(self, h: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> bool:
+        """Whether the kernels may write k and v of the rows h to these stores."""
+        shape = (self.dims.num_kv_heads, h.shape[0], self.dims.head_dim)
+        return (k.dtype is v.dtype is torch.bfloat16 and k.shape == v.shape == shape and K.plain((k, v), ())
+                and k.device == h.device and k.data_ptr() % 16 == v.data_ptr() % 16 == 0)
+
+    def _qkv_into(self, l: int, x: torch.Tensor, pos: torch.Tensor, q, k, v) -> None:
+        """q, k, v of layer l from its normed input rows x, written to the
+        given bf16 tensors [..., n, H, d] (q, v as they are; any strides whose
+        rows of d elements are contiguous)."""
+        dims, w = self.dims, self.layers[l]
+        d, nq, nk = dims.head_dim, dims.num_q_heads * dims.head_dim, dims.num_kv_heads * dims.head_dim
+        wqkv = K.joined(w["wq"], w["wk"], w["wv"])
+        if wqkv is not None:
+            y = torch.nn.functional.linear(x, wqkv)
+            p, ld = y.data_ptr(), (nq + 2 * nk,) * 3
+            src = (p, p + 2 * nq, p + 2 * (nq + nk))
+        else:
+            y = [torch.nn.functional.linear(x, w[n]) for n in ("wq", "wk", "wv")]
+            src, ld = [t.data_ptr() for t in y], (nq, nk, nk)
+        K.qkv_post(*src, ld, [t.data_ptr() for t in (q, k, v)], [s for t in (q, k, v) for s in t.stride()[-3:-1]],
+                   w["q_norm"], w["k_norm"], self.inv_freq, pos, dims.num_q_heads, dims.num_kv_heads, d,
+                   dims.rms_eps)
+
+    def _block(self, l: int, h: torch.Tensor, attn: torch.Tensor):
+        """Layer l after its attention: the residual stream before the MLP's
+        output is added (a tensor of its own), and that output (bf16)."""
+        dims, w = self.dims, self.layers[l]
+        linear = torch.nn.functional.linear
+        a = attn if attn.dtype is torch.bfloat16 else K.to_bf16(attn)
+        h, x = K.add_rms_norm(h, linear(a.flatten(-2), w["wo"]), w["post_norm"], dims.rms_eps)
+        w_gu = K.joined(w["w_gate"], w["w_up"])
+        if w_gu is not None:
+            y = K.silu_mul_joined(linear(x, w_gu))
+        else:
+            y = K.silu_mul(linear(x, w["w_gate"]), linear(x, w["w_up"]))
+        return h, linear(y, w["w_down"])
 
     # -- prefill ----------------------------------------------------------
     @torch.no_grad()
@@ -142,14 +235,22 @@ class RandomDecoder:
         pos = torch.arange(tokens.shape[0], device=self.device)
         h = self.embed[tokens].float()
         for l in range(dims.num_layers):
-            q, k, v = self.qkv(l, h, pos)                   # [T_p, H, d]
-            k_out[l].copy_(k.transpose(0, 1))
-            v_out[l].copy_(v.transpose(0, 1))
+            kl, vl = k_out[l], v_out[l]                     # [Hkv, T_p, d]
+            if type(self).qkv is RandomDecoder.qkv and self._kernels(l, h, pos) and self._store_ok(h, kl, vl):
+                # straight into the stores
+                q = torch.empty((h.shape[0], dims.num_q_heads, dims.head_dim), dtype=torch.bfloat16, device=h.device)
+                self._qkv_into(l, K.rms_norm(h, self.layers[l]["in_norm"], dims.rms_eps), pos, q, kl.transpose(0, 1),
+                               vl.transpose(0, 1))
+                kh, vh = kl[None], vl[None]
+            else:
+                q, k, v = self.qkv(l, h, pos)               # [T_p, H, d]
+                kl.copy_(k.transpose(0, 1))
+                vl.copy_(v.transpose(0, 1))
+                kh, vh = k.transpose(0, 1)[None], v.transpose(0, 1)[None]
             qh = q.transpose(0, 1)[None]                    # [1, Hq, T_p, d]
-            kh = k.transpose(0, 1).repeat_interleave(G, dim=0)[None]
-            vh = v.transpose(0, 1).repeat_interleave(G, dim=0)[None]
-            a = torch.nn.functional.scaled_dot_product_attention(qh, kh, vh, is_causal=True, scale=self.sm_scale)
-            h = self.block_out(l, h, a[0].transpose(0, 1).float())
+            a = torch.nn.functional.scaled_dot_product_attention(qh, kh, vh, is_causal=True, scale=self.sm_scale,
+                                                                 enable_gqa=G > 1)
+            h = self.block_out(l, h, a[0].transpose(0, 1).contiguous())
         return self.logits(h[-1])
 
 

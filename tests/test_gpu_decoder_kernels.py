@@ -1,0 +1,161 @@
+"""The decoder's kernels against the torch expressions they stand in for.
+
+Both compute in fp32 with the same element operations and round to bf16 at the
+same places; only the order of a row's sum differs.  A sum of D squares in
+another order moves rms by at most about D 2^-24 relative, far below the
+spacing of bf16, so a bf16 output differs by one unit in the last place at
+most (2^-7 relative, at a rounding boundary) -- after RoPE, by one unit of the
+larger of the two rotated terms.
+"""
+import pytest
+import torch
+
+from paper_2605_30574_gb300 import build as B
+from paper_2605_30574_gb300 import decoder as K
+from paper_2605_30574_gb300.model import DecoderDims, RandomDecoder, _rms_norm
+
+pytestmark = pytest.mark.gpu
+ULP = 2.0 ** -7
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    B.build()
+
+
+def gen(seed=0):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return g
+
+
+def randn(g, *shape, dtype=torch.float32):
+    return torch.randn(*shape, generator=g, device="cuda").to(dtype)
+
+
+def close(got, want, scale=None):
+    got, want = got.float(), want.float()
+    bound = ULP * (want.abs() if scale is None else scale.float()) + 1e-30
+    assert torch.equal(got.isnan(), want.isnan())
+    ok = ((got - want).abs() <= bound) | got.isnan() | (got == want)
+    assert bool(ok.all()), float(((got - want).abs() / bound).nan_to_num().max())
+
+
+# one thread's row, a ragged vector tail, no vectors, the last row kept in
+# registers, the first that is not, one more than that
+@pytest.mark.parametrize("rows,D", [(1, 4), (3, 36), (2, 37), (5, 1000), (7, 4096), (2, 4100), (2, 8209)])
+def test_norms_and_additions(rows, D):
+    g = gen(D)
+    h, o, w = randn(g, rows, D), randn(g, rows, D, dtype=torch.bfloat16), randn(g, D, dtype=torch.bfloat16)
+    close(K.rms_norm(h, w, 1e-6), _rms_norm(h, w, 1e-6).to(torch.bfloat16))
+    h2, x = K.add_rms_norm(h, o, w, 1e-6)
+    assert torch.equal(h2, h + o.float())
+    close(x, _rms_norm(h2, w, 1e-6).to(torch.bfloat16))
+    assert torch.equal(K.add_(h.clone(), o), h + o.float())
+    assert torch.equal(K.to_bf16(h), h.to(torch.bfloat16))
+    # rows that hold an infinity, a NaN, only zeros
+    h[0, 0] = float("inf")
+    h[-1, -1] = float("nan")
+    close(K.rms_norm(h, w, 1e-6), _rms_norm(h, w, 1e-6).to(torch.bfloat16))
+    assert not K.rms_norm(torch.zeros_like(h), w, 1e-6).any()
+
+
+@pytest.mark.parametrize("rows,F", [(1, 4), (3, 260), (2, 1023), (2, 1028), (70000, 8)])
+def test_silu_product(rows, F):
+    y = randn(gen(F), rows, 2 * F, dtype=torch.bfloat16) * 8
+    y[0, 0], y[-1, 1] = float("-inf"), -200.0
+    gate, up = y[:, :F].contiguous(), y[:, F:].contiguous()
+    want = (torch.nn.functional.silu(gate.float()) * up.float()).to(torch.bfloat16)
+    close(K.silu_mul_joined(y), want)
+    close(K.silu_mul(gate, up), want)
+
+
+def both(model, h, pos):
+    """qkv through the kernels and through torch (which a gradient asks for)."""
+    assert model._kernels(0, h, pos)
+    ours = model.qkv(0, h, pos)
+    hg = h.clone().requires_grad_()
+    assert not model._kernels(0, hg, pos)
+    return ours, [t.detach() for t in model.qkv(0, hg, pos)]
+
+
+@pytest.mark.parametrize("hq,hkv,d,D,F,rows", [(1, 1, 64, 64, 100, 1), (7, 1, 128, 260, 96, 5), (8, 2, 64, 256, 512, 33),
+                                               (12, 4, 256, 520, 36, 9), (32, 8, 128, 4096, 384, 40)])
+def test_layer_pieces(hq, hkv, d, D, F, rows):
+    model = RandomDecoder(DecoderDims(1, hq, hkv, d, D, F, 77), seed=1)
+    g = gen(d)
+    w = model.layers[0]
+    for n in ("in_norm", "q_norm", "k_norm", "post_norm"):
+        w[n].copy_(1 + 0.1 * randn(g, w[n].numel()))
+    h = randn(g, rows, D)
+    pos = torch.randint(0, 100000, (rows,), generator=g, device="cuda")
+    assert K.joined(w["wq"], w["wk"], w["wv"]) is not None and K.joined(w["w_gate"], w["w_up"]) is not None
+
+    def check():
+        (q, k, v), (qt, kt, vt) = both(model, h, pos)
+        # the projections' own sums may round to the next bf16, which the
+        # head's norm then scales: a few units of the head's largest values
+        for a, b in ((q, qt), (k, kt), (v, vt)):
+            assert a.is_contiguous() and a.shape == b.shape and a.dtype is b.dtype
+            close(a, b, scale=2 * b.abs().amax(-1, keepdim=True).expand_as(b))
+        attn = randn(g, rows, hq, d)
+        want = model.block_out(0, h.clone().requires_grad_(), attn).detach()
+        for a in (attn, attn.to(torch.bfloat16)):
+            got = model.block_out(0, h, a)
+            assert (got - want).abs().max() <= 4 * ULP * (want - h).abs().max()
+        lt = model.logits(h.clone().requires_grad_()).detach()
+        close(model.logits(h), lt, scale=lt.abs().amax(-1, keepdim=True).expand_as(lt))
+        close(model.logits(h[0]), lt[0], scale=lt[0].abs().amax().expand_as(lt[0]))
+
+    check()
+    # weights of one's own: the matrices are no longer one
+    w["wk"], w["w_up"] = w["wk"] * 2, w["w_up"].clone()
+    assert K.joined(w["wq"], w["wk"], w["wv"]) is None and K.joined(w["w_gate"], w["w_up"]) is None
+    check()
+    # further leading dimensions, other position types
+    q1, k1, v1 = model.qkv(0, h[None].expand(2, rows, D).contiguous(), pos.int()[None].expand(2, rows).contiguous())
+    q0, k0, v0 = model.qkv(0, h, pos.float())
+    for a, b in ((q1, q0), (k1, k0), (v1, v0)):
+        close(a[1], b, scale=2 * b.abs().amax(-1, keepdim=True).expand_as(b))
+
+
+def test_rope_angles_match_torch_bit_for_bit():
+    """With unit rows (rms 1 exactly) only the rotation is left, whose
+    operations and order are torch's."""
+    model = RandomDecoder(DecoderDims(1, 1, 1, 128, 128, 8, 8), seed=0)
+    w = model.layers[0]
+    eye = torch.eye(128, device="cuda", dtype=torch.bfloat16)
+    for n in ("wq", "wk", "wv"):
+        w[n].copy_(eye)
+    h = torch.ones(300, 128, device="cuda") * (torch.arange(128, device="cuda") % 2 * 2 - 1)
+    pos = torch.arange(300, device="cuda") * 337
+    (q, k, v), (qt, kt, vt) = both(model, h, pos)
+    assert torch.equal(v, vt)
+    assert (q != qt).float().mean() < 1e-3 and (k != kt).float().mean() < 1e-3
+    close(q, qt, scale=torch.ones_like(qt))
+
+
+def test_transforms_modes_and_other_types_take_the_torch_path():
+    model = RandomDecoder(DecoderDims(1, 4, 2, 64, 128, 64, 50), seed=0)
+    h, pos = randn(gen(), 6, 128), torch.arange(6, device="cuda")
+    want = model.qkv(0, h, pos)[0]
+    assert not model._kernels(0, h.double(), pos) and not model._kernels(0, h[:0], pos[:0])
+    assert not model._kernels(0, h, pos[:1]) and not model._kernels(0, h.t().contiguous().t(), pos)
+    with torch.autocast("cuda", dtype=torch.float16):
+        assert not model._kernels(0, h, pos)
+    per_row = torch.func.vmap(lambda r, p: model.qkv(0, r[None], p[None])[0][0])(h, pos)
+    close(per_row, want, scale=2 * want.abs().amax(-1, keepdim=True).expand_as(want))
+    _, tangent = torch.func.jvp(lambda x: model.logits(x), (h,), (h,))
+    assert tangent.abs().max() > 0
+
+
+@pytest.mark.parametrize("hq,hkv,d,T", [(1, 1, 64, 1), (6, 2, 128, 77), (4, 4, 256, 130)])
+def test_prefill_into_stores_and_into_copies(hq, hkv, d, T):
+    """Straight into contiguous bf16 stores, and through copies into others."""
+    model = RandomDecoder(DecoderDims(2, hq, hkv, d, 192, 320, 60), seed=2)
+    tokens = torch.randint(0, 60, (T,), generator=gen(T), device="cuda")
+    k, v = (torch.zeros(2, hkv, T, d, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    kf, vf = (torch.zeros(2, hkv, T, d, device="cuda") for _ in range(2))
+    want = model.prefill(tokens, kf, vf)
+    got = model.prefill(tokens, k, v)
+    assert torch.equal(k.float(), kf) and torch.equal(v.float(), vf) and torch.equal(got, want)
