@@ -426,16 +426,14 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
         if (tc_keys > 0) p.nsd = std::min(max_splits, (d->delta_max + tc_keys - 1) / tc_keys);
     }
     {
-        // Generated-span items: (sequence, kv head, row chunk, key split).
-        // Split so every resident warp gets about two items, but keep at
-        // least 64 keys per split.  Every split costs a partial state to
-        // write and merge; the prompt-span pass queued behind this one fills
-        // the SMs its last warps leave idle, so few splits pay off even
-        // where the items do not share out evenly over the warps.
-        const int G = sh.num_q_heads / sh.num_kv_heads;
-        const int gt = G % 4 == 0 ? 4 : (G % 2 == 0 ? 2 : 1);
-        const long base_items = long(d->B) * sh.num_kv_heads * (G / gt);
-        const long want = 2L * splice::generated_span_resident_warps(sh.head_dim);
+        // Generated-span items: (sequence, kv head, key split).  Split so
+        // every resident warp gets about two items, but keep at least 64 keys
+        // per split.  Every split costs a partial state to write and merge;
+        // the prompt-span pass queued behind this one fills the SMs its last
+        // warps leave idle, so few splits pay off even where the items do not
+        // share out evenly over the warps.
+        const long base_items = long(d->B) * sh.num_kv_heads;
+        const long want = 2L * splice::generated_span_resident_warps(sh.head_dim, p.G);
         int ns = int(std::min<long>(splice::kMaxSuffixSplits, std::max<long>(1, (want + base_items - 1) / base_items)));
         ns = std::min(ns, std::max(1, s_vis / 64));
         p.nss = s_vis > 0 ? ns : 0;
@@ -458,8 +456,8 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
     // first: its short run and its tail (part of the SMs idle while its last
     // items finish) are filled by the generated-span pass's run-time claimed
     // items.  So does a prompt-span pass with more than
-    // kPrefixFirstGenRatio times the generated-span pass's keys (x row
-    // chunks): the generated-span pass's short items then fill its tail.
+    // kPrefixFirstGenRatio times the generated-span pass's keys: the
+    // generated-span pass's short items then fill its tail.
     // With per-launch timing on, the events between the launches serialise
     // everything.
     const bool gs_work = p.nss > 0;
@@ -471,7 +469,7 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
         (long(p.n_span_tiles) * ((p_vis + box - 1) / box) +
          long(p.n_tiles - p.n_span_tiles) * (p.nsd ? (d->delta_max + box - 1) / box : 0)) *
         sh.num_kv_heads * box;
-    const long gs_keys = long(d->B) * sh.num_kv_heads * (p.G / (p.G % 4 == 0 ? 4 : (p.G % 2 == 0 ? 2 : 1))) * s_vis;
+    const long gs_keys = long(d->B) * sh.num_kv_heads * s_vis;
     const bool prefix_first =
         prefix_launched &&
         (d->pass_order == 1 ||

@@ -1,11 +1,13 @@
-// Generated-span pass (CUDA cores): attention of the G query rows of one
-// (sequence, kv head) over that sequence's own generated-span K/V (§3: the
-// decode step attends over the prompt span and the t generated entries).
+// Generated-span pass on CUDA cores, for one query row per kv head (and two or
+// four of 256 dims; k_suffix_mma.cu has the rest and the rule is at the end
+// of this file): attention of the G query rows of one (sequence, kv head) over
+// that sequence's own generated-span K/V (§3: the decode step attends over the
+// prompt span and the t generated entries).
 //
 // HBM-bound streaming kernel:
-//   * persistent warps walking work items (sequence, kv head, row chunk, key
-//     split) and, inside an item, blocks of 16 keys: a fixed stream per warp
-//     when this pass goes first, items claimed at run time (one ahead) when
+//   * persistent warps walking work items (sequence, kv head, key split) and,
+//     inside an item, blocks of 16 keys: a fixed stream per warp when this
+//     pass goes first, items claimed at run time (one ahead) when
 //     it runs behind the prompt-span pass, so warps that start late (on SMs
 //     that pass still holds) simply take fewer; the issue cursor decodes
 //     each item once and hands it to the consumer through a per-warp ring;
@@ -34,34 +36,19 @@
 
 #include <cmath>
 
-#include "splice_internal.h"
+#include "gs_common.cuh"
 #include "tc_ptx.cuh"
 
 namespace splice {
 namespace {
 
-constexpr unsigned kFull = 0xffffffffu;
-constexpr float kTau = 8.0f;
-constexpr unsigned kErrWaitGs = 0x10, kErrWaitGsDrain = 0x80;
+using namespace gs;
 
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
+constexpr unsigned kErrWaitGs = 0x10, kErrWaitGsDrain = 0x80;
 
 // bf16 pair word -> (even dim, odd dim) as fp32
 __device__ __forceinline__ float2 unpack2(uint32_t w) {
     return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-
-// Generated-span K/V is read once: the copy marks its L2 lines first to be
-// evicted, so the streamed bytes do not push out the partial states the
-// merge reads right after.
-__device__ __forceinline__ uint64_t l2_evict_first_policy() {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
 }
 
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, uint64_t pol) {
@@ -72,37 +59,6 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
         : "memory");
 }
 
-__device__ __forceinline__ unsigned ld_relaxed_gpu(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-
-// The merge of a row's two partial states -- the prompt-span pass's (when
-// has_span) and this pass's -- with a ZERO span's closed form, in exactly
-// the operations and order of the merge kernel for a row of at most two
-// states (merge_row.cuh): the same bits.  Returns the factor of the
-// weighted sum (0 for a row with nothing live) and the two weights.
-__device__ __forceinline__ float merge_two_weights(bool has_span, float2 ml_span, float m_gen, float l_gen,
-                                                   bool zero_span, int n_zero, float* w_span, float* w_gen) {
-    const bool live_s = has_span && ml_span.y > 0.f, live_g = l_gen > 0.f;
-    float M = fmaxf(live_s ? ml_span.x : -INFINITY, live_g ? m_gen : -INFINITY);
-    if (zero_span) M = fmaxf(M, 0.f);
-    *w_span = live_s ? exp2f(ml_span.x - M) : 0.f;
-    *w_gen = live_g ? exp2f(m_gen - M) : 0.f;
-    float den = __fadd_rn(has_span ? __fmul_rn(*w_span, ml_span.y) : 0.f, __fmul_rn(*w_gen, l_gen));
-    if (zero_span) den = fmaf(float(n_zero), exp2f(0.f - M), den);
-    return den > 0.f ? 1.f / den : 0.f;
-}
-
-__device__ __forceinline__ float merge_two(bool has_span, float w_span, float o_span, float w_gen, float o_gen,
-                                           float inv) {
-    float acc = 0.f;
-    if (has_span && w_span != 0.f) acc = fmaf(w_span, o_span, acc);
-    if (w_gen != 0.f) acc = fmaf(w_gen, o_gen, acc);
-    return __fmul_rn(acc, inv);
-}
-
 // The same without a cache hint: the query rows are read again by the
 // prompt-span pass of the call.
 __device__ __forceinline__ void bulk_copy_plain(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -110,10 +66,6 @@ __device__ __forceinline__ void bulk_copy_plain(uint32_t dst, const void* src, u
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
-
-// Items a warp may leave unmerged until its end (with P.gs_merge): those
-// that end before the prompt-span pass has completed.
-constexpr int kPend = 8;
 
 template <int D, int GT>
 struct GS {
@@ -145,53 +97,6 @@ struct GS {
     static_assert(NV < LPK || NV == VPL * LPK, "every logit of a group owned by one lane");
     static_assert(LPK % GT == 0, "the logits of a lane belong to one query row");
 };
-
-// n / d for 0 <= n < 2^31 by a multiply and a shift, for a divisor fixed
-// per launch (Granlund and Montgomery, "Division by invariant integers using
-// multiplication", 1994, the round-up method): with s = ceil(log2 d) and
-// m = floor(2^32 (2^s - d) / d) + 1, n / d = (umulhi(n, m) + n) >> s; the
-// sum stays below 2^32 because umulhi(n, m) < n < 2^31.
-struct FastDiv {
-    uint32_t d, m, s;
-    __device__ explicit FastDiv(int divisor) : d(uint32_t(divisor)), m(1), s(0) {
-        while ((1u << s) < d) ++s;
-        m = uint32_t((((uint64_t(1) << s) - d) << 32) / d + 1);
-    }
-    __device__ __forceinline__ int div(int n) const { return int((__umulhi(uint32_t(n), m) + uint32_t(n)) >> s); }
-};
-
-struct ItemDivs {
-    FastDiv nss, n_rc, hkv;
-};
-
-// One work item: where its rows and keys are.  The issue cursor decodes
-// each item once and hands it to the consumer through the warp's ring
-// (eight ints, idx -1 for the end of the walk).
-struct Item {
-    int idx, s, h, rc, split, k0, k1, nblk;
-};
-
-// Work item idx = ((sequence * Hkv + kv head) * row chunks + row chunk) *
-// splits + key split.
-__device__ __forceinline__ void item_of(const AttnParams& P, const ItemDivs& dv, int idx, Item& it) {
-    it.idx = idx;
-    int rem = dv.nss.div(idx);
-    it.split = idx - rem * P.nss;
-    const int sh = dv.n_rc.div(rem);
-    it.rc = rem - sh * int(dv.n_rc.d);
-    it.s = dv.hkv.div(sh);
-    it.h = sh - it.s * P.Hkv;
-    it.k0 = P.s_lo + it.split * P.s_chunk;
-    it.k1 = min(P.s_hi, it.k0 + P.s_chunk);
-    it.nblk = it.k1 > it.k0 ? (it.k1 - it.k0 + 15) / 16 : 0;
-}
-
-// Offset (in elements) of the generated-span K/V rows of (sequence, kv head)
-// at this layer.
-template <int D>
-__device__ __forceinline__ size_t span_base(const AttnParams& P, int s, int h) {
-    return ((size_t(s) * P.N + P.layer) * P.Hkv + h) * size_t(P.T) * D;
-}
 
 template <int D, int GT>
 __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
@@ -301,14 +206,14 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
     // item it takes, decoded (then the end, idx -1), for the consumer.  It
     // runs two blocks ahead and every item has a block (the host keeps at
     // least 64 keys per split), so it is at most two items ahead ----
-    const ItemDivs dv{FastDiv(P.nss), FastDiv(P.G / GT), FastDiv(P.Hkv)};
+    const ItemDivs dv{FastDiv(P.nss), FastDiv(P.Hkv)};
     Item iss;
     int iss_idx = first_item < n_items ? first_item : -1, iss_b = 0, recorded = 0;
     bool iss_ok = false;
     auto record = [&](const Item& e) {
         if (lane == 0) {
-            ring[2 * (recorded & 3)] = make_int4(e.idx, e.s, e.h, e.rc);
-            ring[2 * (recorded & 3) + 1] = make_int4(e.split, e.k0, e.k1, e.nblk);
+            ring[2 * (recorded & 3)] = make_int4(e.idx, e.s, e.h, e.split);
+            ring[2 * (recorded & 3) + 1] = make_int4(e.k0, e.k1, e.nblk, 0);
         }
         ++recorded;
     };
@@ -347,7 +252,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             tc::mbar_arrive_expect_tx(bar0 + 8 * stg, 2 * bytes + (first ? C::QROWS : 0u));
             if (first)
                 bulk_copy_plain(wbase + C::OFF_Q + (iss_items & 1) * C::QROWS,
-                                P.q + (size_t(iss.s) * P.Hq + iss.h * P.G + iss.rc * GT) * D, C::QROWS, bar0 + 8 * stg);
+                                P.q + (size_t(iss.s) * P.Hq + iss.h * GT) * D, C::QROWS, bar0 + 8 * stg);
             if (bytes) {
                 bulk_copy(dst, P.ks + iss_base + size_t(j) * D, bytes, bar0 + 8 * stg, pol);
                 bulk_copy(dst + C::BK * C::ROW, P.vs + iss_base + size_t(j) * D, bytes, bar0 + 8 * stg, pol);
@@ -388,7 +293,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
         const int4 e0 = ring[2 * (taken & 3)];
         if (e0.x < 0) break;
         const int4 e1 = ring[2 * (taken & 3) + 1];
-        const Item it{e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+        const Item it{e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z};
         // merges in this pass: the rows' source (a ZERO row needs no
         // prompt-span state) and, until it has been seen set, the prompt-span
         // pass's completion flag, read now and used at the item's end
@@ -463,7 +368,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             const int jb = it.k0 + b * 16;
             if (tail && b == it.nblk - 1) {
                 // the step's own entry: its row of the stage from registers,
-                // and (once per (sequence, kv head)) into the store
+                // and into the store
                 const int rj = P.s_hi - 1 - jb;
                 const size_t ent = ((size_t(it.s) * P.N + P.layer) * P.Hkv + it.h) * size_t(P.T) + (P.s_hi - 1);
 #pragma unroll
@@ -473,8 +378,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
                         const bool isk = c < D / 8;
                         const int cc = isk ? c : c - D / 8;
                         *reinterpret_cast<uint4*>((isk ? kst : vst) + rj * C::ROW + cc * 16) = nkv[i];
-                        if (it.rc == 0)
-                            reinterpret_cast<uint4*>(isk ? P.ks_w : P.vs_w)[ent * (D / 8) + cc] = nkv[i];
+                        reinterpret_cast<uint4*>(isk ? P.ks_w : P.vs_w)[ent * (D / 8) + cc] = nkv[i];
                     }
                 }
                 __syncwarp();
@@ -625,7 +529,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             if (merge_here && has_span) {
 #pragma unroll
                 for (int g = 0; g < GT; ++g) {
-                    const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;   // split 0's slot
+                    const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;   // split 0's slot
                     ml_span[g] = __ldcg(P.ws_ml + row);
                     const float* sp = P.ws_o + row * D + dim0;
                     if constexpr (F == 2) {
@@ -697,7 +601,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             const bool zero_span = !has_span && P.p_hi > P.p_lo;
 #pragma unroll
             for (int g = 0; g < GT; ++g) {
-                const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;
+                const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;
                 // the row's (m, l) as lane 0 would store it: the lanes' row
                 // sums can differ in the last bit (each lane adds its pair's
                 // two terms in its own order)
@@ -722,7 +626,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             const int slot = kMaxPrefixSplits + it.split;
 #pragma unroll
             for (int g = 0; g < GT; ++g) {
-                const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;
+                const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;
                 const size_t idx2 = size_t(slot) * P.B * P.Hq + row;
                 float* op = P.ws_o + idx2 * D + dim0;
                 if constexpr (F == 2) {
@@ -766,7 +670,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
                     item_of(P, dv, pend[k], it);
 #pragma unroll
                     for (int g = 0; g < GT; ++g) {
-                        const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;
+                        const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;
                         const size_t gen = size_t(kMaxPrefixSplits) * P.B * P.Hq + row;
                         const float2 ml_gen = __ldcg(P.ws_ml + gen), ml_span = __ldcg(P.ws_ml + row);
                         float og[F], os[F];
@@ -826,31 +730,38 @@ int launch_gs_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap_
 
 }  // namespace
 
-int generated_span_resident_warps(int d) {
+// The FMA kernel above for one query row per kv head (d = 64, 128, 256) and
+// for two or four of 256 dims; the tensor-core kernel for the rest.  At one
+// row the FMA kernel has less to do per key (140 x 8 heads of 128 dims x 500
+// keys: 44.7 us against 45.6); rows of 256 dims leave the tensor-core kernel
+// five or six warps per SM, whose longer chains per block two or four rows do
+// not repay (1152 x 4 heads x 150 keys, two rows: 118 us against 125; a
+// Gemma-3-4B-shaped layer 123 against 132).  Everywhere else all rows of a kv
+// head share one read of K and V there, and even at four rows of 128 dims,
+// where both kernels read once, it is faster (512 x 8 heads x 512 keys: 173 us
+// against 168; eight rows, 300 x 8 heads x 277 keys: 110 against 58).
+static bool fma_kernel(int d, int G) { return G == 1 || (d == 256 && (G == 2 || G == 4)); }
+
+int generated_span_resident_warps(int d, int G) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // two 4-warp CTAs per SM (d <= 128), three 2-warp CTAs per SM (d = 256)
-    return sms * (d == 256 ? 6 : 8);
+    // FMA kernel: two 4-warp CTAs per SM (d <= 128), three 2-warp CTAs per SM (d = 256)
+    return sms * (fma_kernel(d, G) ? (d == 256 ? 6 : 8) : gs::mma_warps_per_sm(d, G));
 }
 
 bool generated_span_can_merge(int d, int G) {
-    const int gt = G % 4 == 0 ? 4 : (G % 2 == 0 ? 2 : 1);
-    return gt * d <= 512;   // GT * F <= 16 in gs_kernel, F = d / 32
+    return fma_kernel(d, G) ? G * d <= 512 : gs::mma_can_merge(d, G);   // GT * F <= 16 in gs_kernel, F = d / 32
 }
 
 int launch_generated_span(const AttnParams& p, void* stream, bool overlap_previous) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int gt = p.G % 4 == 0 ? 4 : (p.G % 2 == 0 ? 2 : 1);
-    const long n_items = long(p.B) * p.Hkv * (p.G / gt) * p.nss;
+    const long n_items = long(p.B) * p.Hkv * p.nss;
     if (n_items == 0) return 0;
-    switch (p.D * 8 + gt) {
+    if (!fma_kernel(p.D, p.G)) return gs::launch_mma(p, st, overlap_previous);
+    switch (p.D * 8 + p.G) {
         case 64 * 8 + 1: return launch_gs_t<64, 1>(p, int(n_items), st, overlap_previous);
-        case 64 * 8 + 2: return launch_gs_t<64, 2>(p, int(n_items), st, overlap_previous);
-        case 64 * 8 + 4: return launch_gs_t<64, 4>(p, int(n_items), st, overlap_previous);
         case 128 * 8 + 1: return launch_gs_t<128, 1>(p, int(n_items), st, overlap_previous);
-        case 128 * 8 + 2: return launch_gs_t<128, 2>(p, int(n_items), st, overlap_previous);
-        case 128 * 8 + 4: return launch_gs_t<128, 4>(p, int(n_items), st, overlap_previous);
         case 256 * 8 + 1: return launch_gs_t<256, 1>(p, int(n_items), st, overlap_previous);
         case 256 * 8 + 2: return launch_gs_t<256, 2>(p, int(n_items), st, overlap_previous);
         case 256 * 8 + 4: return launch_gs_t<256, 4>(p, int(n_items), st, overlap_previous);

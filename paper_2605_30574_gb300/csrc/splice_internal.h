@@ -28,7 +28,7 @@ constexpr int kPrefixSplitKeys = 1024;
 // keys (summed over its items) per SM.
 constexpr int kPrefixFirstKeysPerSm = 3072;
 // It also goes first when its keys exceed kPrefixFirstGenRatio x the
-// generated-span pass's (keys x row chunks).
+// generated-span pass's.
 constexpr int kPrefixFirstGenRatio = 2;
 // Group source flag: the group reads the delta-encoded rows of a donor slot
 // (group_src = kGroupDelta | (SPLICE_SRC_DONOR0 + slot)).
@@ -154,7 +154,7 @@ int launch_append(const uint16_t* kn, const uint16_t* vn, uint16_t* ks, uint16_t
 // flag (sched[4]) and fenced, waits for it only before it exits, and lets
 // its own dependents launch only once its work is done.
 int launch_generated_span(const AttnParams& p, void* stream, bool overlap_previous);
-int generated_span_resident_warps(int d);
+int generated_span_resident_warps(int d, int G);
 // Whether the generated-span pass is built with its merge path for head
 // dim d and GQA group G (AttnParams::gs_merge may be set only then).
 bool generated_span_can_merge(int d, int G);
@@ -191,7 +191,7 @@ int prefix_tc_splits(int d, int p_vis, int max_splits, int* bounds);
 int launch_prefix_tc(const AttnParams& p, const void* maps, const int* bounds, int delta_keys, void* stream,
                      bool overlap_previous);
 
-// Delta encoding of every stored donor span (one CTA per span): bits of the
+// Delta encoding of every stored donor span: bits of the
 // positions whose K or V row differs from the clean span, their count, and
 // the donor rows at those positions compacted to the front of the span's
 // rows in the delta store (the remaining rows zeroed).
