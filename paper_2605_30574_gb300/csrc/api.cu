@@ -409,7 +409,8 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
     int tc_split = 0, tc_keys = 0;
     int bounds[splice::kMaxPrefixSplits + 1] = {0};
     if (p_vis > 0) {
-        tc_split = splice::prefix_tc_splits(sh.head_dim, p_vis, max_splits, bounds);
+        tc_split = splice::prefix_tc_splits(sh.head_dim, p_vis, max_splits, long(d->plan.tile_bound) * sh.num_kv_heads,
+                                            d->sms, bounds);
         tc_keys = bounds[1];           // the longest split
     }
     p.nsp = tc_split;

@@ -45,6 +45,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "splice_internal.h"
@@ -1020,6 +1021,13 @@ int launch_d(const TcParams& tp, const CUtensorMap* m, cudaStream_t st, bool ove
     return int(cudaLaunchKernelEx(&cfg, prefix_tc_kernel<D, SHORT>, m[0], m[1], m[2], m[3], m[4], m[5], tp));
 }
 
+// What a small launch is made of, measured on launches of one item per SM:
+// a key block (128 keys; 64 for d = 256), an item beside its blocks (its first
+// loads, its last P V, its partial states), the merge launch that several
+// splits need where one leaves the merge to the generated-span pass, and the
+// rate at which larger launches stream.
+constexpr double kBlockUs = 0.96, kBlockUs256 = 0.8, kItemUs = 2.2, kMergeUs = 2.5, kStreamBytesPerUs = 6.0e6;
+
 }  // namespace
 
 // 2D view [rows][d] of a bf16 store; box = 64 elements x box_rows rows, 128-byte swizzle.
@@ -1041,12 +1049,13 @@ int prefix_tc_box_rows(int d) {
     return d == 64 ? Cfg<64>::BN : (d == 128 ? Cfg<128>::BN : Cfg<256>::BN);
 }
 
-int prefix_tc_splits(int d, int p_vis, int max_splits, int* bounds) {
-    // Splits depend only on the visible span length (and the cap), so a
-    // row's arithmetic never depends on which other rows share its tile or
-    // launch.  Every item gathers its tile's queries and stores its partial
-    // states, so long items move fewer bytes; but a launch ends as unevenly
-    // as its last items are long.  So a span's first split is
+int prefix_tc_splits(int d, int p_vis, int max_splits, long spans, int sms, int* bounds) {
+    // Splits depend on the visible span length, the cap and the descriptor's
+    // prompts and donor slots (`spans`), never on the cells' L and W, so a
+    // row's arithmetic never depends on which other rows share its tile or on
+    // what they read.  Every item gathers its tile's queries and stores its
+    // partial states, so long items move fewer bytes; but a launch ends as
+    // unevenly as its last items are long.  So a span's first split is
     // kPrefixFirstSplitKeys keys and the rest kPrefixSplitKeys: the
     // split-major item order hands out every span's long first split before
     // the short ones, and the launch ends on short items.  Past the cap, the
@@ -1054,18 +1063,36 @@ int prefix_tc_splits(int d, int p_vis, int max_splits, int* bounds) {
     const int bn = prefix_tc_box_rows(d);
     const int nb = (p_vis + bn - 1) / bn;
     const int first = kPrefixFirstSplitKeys / bn, rest = kPrefixSplitKeys / bn;
-    const int ns_full = nb <= first ? 1 : 1 + (nb - first + rest - 1) / rest;
-    bounds[0] = 0;
-    if (ns_full <= max_splits) {
-        for (int i = 0; i < ns_full; ++i) {
-            const int b = bounds[i] + (i == 0 ? first : rest) * bn;
-            bounds[i + 1] = b < p_vis ? b : p_vis;
+    int ns = nb <= first ? 1 : 1 + (nb - first + rest - 1) / rest;
+    bool even = ns > max_splits;
+    if (even) ns = max_splits;
+    // A launch of fewer than two items per SM lasts as long as a few rounds
+    // of items, not as its bytes take: then the even split of the least
+    // estimated time, if that is less than that of the splits above.  With
+    // one prompt of 2048 keys read by 15 cells (8 kv heads of 128) a layer
+    // takes 15.4 us in four splits and 25.8 in one; of 6000 keys 29 against 34;
+    // one cell's 4096 keys 13.6 in eight against 24.5 in 2048 + 1024 + 1024.
+    if (spans * ns < 2L * sms) {
+        const double bytes_us = double(spans) * p_vis * d * 4 / kStreamBytesPerUs;
+        auto time = [&](int n, double longest) {
+            const double chain = longest * (d == 256 ? kBlockUs256 : kBlockUs) + double((spans * n + sms - 1) / sms) * kItemUs;
+            return std::max(chain, bytes_us + kItemUs) + (n > 1 ? kMergeUs : 0.0);
+        };
+        const int longest = nb < first ? nb : first;
+        double best = even ? time(ns, double((spans * ns + sms - 1) / sms) * ((nb + ns - 1) / ns))
+                           : time(ns, std::max(double(longest), double(spans) * nb / sms + (ns > 1 ? rest / 2 : 0)));
+        for (int n = 1; n <= max_splits && n * kPrefixMinSplitKeys <= p_vis; ++n) {
+            const double t = time(n, double((spans * n + sms - 1) / sms) * ((nb + n - 1) / n));
+            if (t < best) {
+                best = t;
+                ns = n;
+                even = true;
+            }
         }
-        return ns_full;
     }
-    const int ns = max_splits;
+    bounds[0] = 0;
     for (int i = 0; i < ns; ++i) {
-        const int blocks = nb / ns + (i < nb % ns ? 1 : 0);
+        const int blocks = even ? nb / ns + (i < nb % ns ? 1 : 0) : (i == 0 ? first : rest);
         const int b = bounds[i] + blocks * bn;
         bounds[i + 1] = b < p_vis ? b : p_vis;
     }

@@ -31,12 +31,15 @@ __global__ void append_kernel(const uint4* __restrict__ kn, const uint4* __restr
 }
 
 // The partial states of the prompt-span and the generated-span passes (and
-// the ZERO closed form) -> out.  Rows with up to four partials -- the common
-// case -- take a one-round-trip path: for d <= 128 a warp merges two rows,
-// one per half-warp; for d = 256 one row per warp.  Rows with more partials
-// take the general path, a warp per row.
-template <int D>
-__global__ void __launch_bounds__(256, 5) merge_kernel(AttnParams P) {
+// the ZERO closed form) -> out, for calls whose rows have up to NF partials
+// (4 -- the common case --, 8 or 16): every load of a row goes out before any
+// is used, one round trip.  Up to 8 partials of d <= 128, a warp merges two
+// rows, one per half-warp; else one row.  (Rows of more than four partials
+// used to take two dependent round trips, one row of a warp after the other:
+// the delta-mode ladder layer's six 118.5 us against 116.6 now, and a small
+// launch of five 17.6 against 13.1.)
+template <int D, int NF>
+__global__ void __launch_bounds__(256, NF == 4 ? 5 : (NF == 8 ? 2 : 1)) merge_kernel(AttnParams P) {
     // Launched behind the prompt-span pass as a programmatic dependent, this
     // grid may start before that pass has finished: wait for it (and so for
     // the generated-span pass it waited for) before reading any partial.
@@ -45,15 +48,10 @@ __global__ void __launch_bounds__(256, 5) merge_kernel(AttnParams P) {
     const long warp = (long(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const long total = long(P.B) * P.Hq;
-    if constexpr (D <= 128) {
-        const long row0 = 2 * warp;
-        if (row0 >= total) return;
-        if (merge_rows_fast2<D, 4>(P, row0, lane)) return;
-        merge_row(P, row0, lane);
-        if (row0 + 1 < total) merge_row(P, row0 + 1, lane);
+    if constexpr (D <= 128 && NF <= 8) {
+        if (2 * warp < total) merge_rows_group<D, NF, 2>(P, 2 * warp, lane);
     } else {
-        if (warp >= total) return;
-        if (!merge_row_fast<D, 4>(P, warp, lane)) merge_row(P, warp, lane);
+        if (warp < total) merge_row_fast<D, NF>(P, warp, lane);
     }
 }
 
@@ -68,13 +66,22 @@ __global__ void __launch_bounds__(256, 3) merge_kernel4(AttnParams P) {
     const int lane = threadIdx.x & 31;
     const long total = long(P.B) * P.Hq;
     const long row0 = 4 * warp;
-    if (row0 >= total) return;
-    if (merge_rows_group<D, 2, 4>(P, row0, lane)) return;
-    for (long r = row0; r < row0 + 4 && r < total; r += 2)
-        if (!merge_rows_fast2<D, 4>(P, r, lane)) {
-            merge_row(P, r, lane);
-            if (r + 1 < total) merge_row(P, r + 1, lane);
-        }
+    if (row0 < total) merge_rows_group<D, 2, 4>(P, row0, lane);
+}
+
+template <int D, int NF>
+int launch_merge_t(cudaLaunchConfig_t& cfg, long rows, const AttnParams& p) {
+    const long warps = D <= 128 && NF <= 8 ? (rows + 1) / 2 : rows;
+    cfg.blockDim = dim3(256);
+    cfg.gridDim = dim3(unsigned((warps * 32 + 255) / 256));
+    return int(cudaLaunchKernelEx(&cfg, merge_kernel<D, NF>, p));
+}
+
+template <int D>
+int launch_merge_d(cudaLaunchConfig_t& cfg, long rows, int partials, const AttnParams& p) {
+    if (partials <= 4) return launch_merge_t<D, 4>(cfg, rows, p);
+    if (partials <= 8) return launch_merge_t<D, 8>(cfg, rows, p);
+    return launch_merge_t<D, 16>(cfg, rows, p);
 }
 
 }  // namespace
@@ -93,29 +100,26 @@ int launch_append(const uint16_t* kn, const uint16_t* vn, uint16_t* ks, uint16_t
 
 int launch_merge(const AttnParams& p, void* stream, bool overlap_previous) {
     const long rows = long(p.B) * p.Hq;
-    const int block = 256;
-    // at most two partials per row: the prompt-span splits (none for a ZERO
-    // row), the generated-span splits and a delta row's splits
-    const bool four = p.D <= 128 && p.nsp + p.nss + (p.delta_on ? p.nsd : 0) <= 2;
-    const long warps = four ? (rows + 3) / 4 : (p.D <= 128 ? (rows + 1) / 2 : rows);
-    const long threads = warps * 32;
+    // the most partials a row can have: the prompt-span splits (none for a
+    // ZERO row), the generated-span splits and a delta row's splits
+    const int partials = p.nsp + p.nss + (p.delta_on ? p.nsd : 0);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned((threads + block - 1) / block));
-    cfg.blockDim = dim3(block);
     cfg.stream = static_cast<cudaStream_t>(stream);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap_previous ? 1 : 0;
-    if (four) {
+    if (p.D <= 128 && partials <= 2) {
+        cfg.blockDim = dim3(256);
+        cfg.gridDim = dim3(unsigned(((rows + 3) / 4 * 32 + 255) / 256));
         if (p.D == 64) return int(cudaLaunchKernelEx(&cfg, merge_kernel4<64>, p));
         return int(cudaLaunchKernelEx(&cfg, merge_kernel4<128>, p));
     }
     switch (p.D) {
-        case 64: return int(cudaLaunchKernelEx(&cfg, merge_kernel<64>, p));
-        case 128: return int(cudaLaunchKernelEx(&cfg, merge_kernel<128>, p));
-        case 256: return int(cudaLaunchKernelEx(&cfg, merge_kernel<256>, p));
+        case 64: return launch_merge_d<64>(cfg, rows, partials, p);
+        case 128: return launch_merge_d<128>(cfg, rows, partials, p);
+        case 256: return launch_merge_d<256>(cfg, rows, partials, p);
         default: return int(cudaErrorInvalidValue);
     }
 }

@@ -56,7 +56,8 @@ __device__ __forceinline__ float merge_weights(const AttnParams& P, int lane, in
     return den > 0.f ? 1.f / den : 0.f;
 }
 
-// Rows with at most NF live partials: every load of the row -- lane i's
+// Rows with at most NF partials (false, and nothing written, for another):
+// every load of the row -- lane i's
 // (m, l) of partial i and this lane's 16-byte slices of o of every partial --
 // is issued before any of them is used, so a row costs one round trip.
 template <int D, int NF>
@@ -183,45 +184,6 @@ __device__ __forceinline__ bool merge_rows_group(const AttnParams& P, long row0,
         }
     }
     return true;
-}
-
-template <int D, int NF>
-__device__ __forceinline__ bool merge_rows_fast2(const AttnParams& P, long row0, int lane) {
-    return merge_rows_group<D, NF, 2>(P, row0, lane);
-}
-
-// Any number of live partials (up to kMaxSplits): weights first, then the o
-// slices.
-__device__ __forceinline__ void merge_row(const AttnParams& P, long row, int lane) {
-    const int s = int(row / P.Hq);
-    const uint8_t code = P.src[s];
-    const RowParts rp = row_parts(P, code);
-    const int n = rp.span + rp.suffix + rp.delta;      // <= kMaxSplits (16)
-    const size_t plane = size_t(P.B) * P.Hq;
-    float2 ml = make_float2(-INFINITY, 0.f);
-    if (lane < n) ml = __ldcg(P.ws_ml + size_t(merge_slot(lane, rp)) * plane + row);
-    float w;
-    const float inv = merge_weights(P, lane, n, code == SPLICE_SRC_ZERO && P.p_hi > P.p_lo, ml, &w);
-    float wall[kMaxSplits];
-#pragma unroll
-    for (int i = 0; i < kMaxSplits; ++i) wall[i] = __shfl_sync(0xffffffffu, w, i);
-    const int c4 = P.D / 4;
-    float4* out = reinterpret_cast<float4*>(P.out + size_t(row) * P.D);
-    for (int c = lane; c < c4; c += 32) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < kMaxSplits; ++i) {
-            if (i < n && wall[i] != 0.f) {
-                const float4 o = __ldcg(reinterpret_cast<const float4*>(
-                                            P.ws_o + (size_t(merge_slot(i, rp)) * plane + row) * P.D) + c);
-                acc.x = fmaf(wall[i], o.x, acc.x);
-                acc.y = fmaf(wall[i], o.y, acc.y);
-                acc.z = fmaf(wall[i], o.z, acc.z);
-                acc.w = fmaf(wall[i], o.w, acc.w);
-            }
-        }
-        out[c] = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
-    }
 }
 
 }  // namespace splice

@@ -17,6 +17,7 @@
 #include <numeric>
 #include <string>
 #include <tuple>
+#include <utility>
 
 #include "splice_internal.h"
 
@@ -60,6 +61,18 @@ std::string build_plan(const splice_model_shape& sh, int P, int Tp, int Dslots, 
     int n_stored = 0;
     for (int k = 0; k < Dslots; ++k)
         if (kinds[k] != SPLICE_DONOR_ZERO) stored[k] = n_stored++;
+
+    std::vector<std::pair<int, int>> reads;             // (prompt, stored index or -1 for the clean span)
+    for (int s = 0; s < B; ++s) {
+        reads.emplace_back(seqs[s].prompt_id, -1);
+        if (stored[seqs[s].donor_slot] >= 0) reads.emplace_back(seqs[s].prompt_id, stored[seqs[s].donor_slot]);
+    }
+    std::sort(reads.begin(), reads.end());
+    plan.tile_bound = 0;
+    for (size_t i = 0, j; i < reads.size(); i = j) {
+        for (j = i; j < reads.size() && reads[j] == reads[i];) ++j;
+        plan.tile_bound += (int(j - i) + plan.seqs_per_tile - 1) / plan.seqs_per_tile;
+    }
 
     plan.src.assign(size_t(plan.num_tables) * B, 0);
     plan.table_group_off.assign(plan.num_tables + 1, 0);

@@ -24,6 +24,9 @@ constexpr int kTileRows = 128;
 // every later one kPrefixSplitKeys (the last possibly fewer).
 constexpr int kPrefixFirstSplitKeys = 2048;
 constexpr int kPrefixSplitKeys = 1024;
+// A launch too small to fill the GPU with those shares a span out evenly, in
+// splits of at least this many keys (see prefix_tc_splits).
+constexpr int kPrefixMinSplitKeys = 512;
 // The call's prompt-span pass goes first when it holds fewer than this many
 // keys (summed over its items) per SM.
 constexpr int kPrefixFirstKeysPerSm = 3072;
@@ -65,6 +68,10 @@ struct Plan {
     std::vector<int32_t> tiles;             // [tiles][4]: group, first, count, (span base << 2) | store kind
     std::vector<int32_t> table_span_tiles;  // [num_tables] tiles of stored-span groups (the rest read delta rows)
     int seqs_per_tile = 0;
+    // Tiles that the prompts' clean and stored donor spans can have at most
+    // in a table, whatever the cells' L and W: the launch-size estimate behind
+    // the span splits.
+    int tile_bound = 0;
 
     int table_of(int layer, int step) const;
 };
@@ -174,10 +181,12 @@ int launch_wait_timeout(unsigned* err, unsigned long long limit_ns, void* stream
 // Tensor-core prompt-span pass.  A tensor map is a 128-byte CUtensorMap.
 int make_kv_tensor_map(void* out_map, const void* base, long rows, int d, int box_rows);
 int prefix_tc_box_rows(int d);
-// Key splits of a visible span of p_vis keys: returns their number n (at
+// Key splits of a visible span of p_vis keys in a launch of about `spans`
+// (tile, kv head) pairs on `sms` multiprocessors: returns their number n (at
 // most max_splits) and writes bounds[0 .. n], 0 = bounds[0] < ... <
-// bounds[n] = p_vis, every inner bound a multiple of the key block.
-int prefix_tc_splits(int d, int p_vis, int max_splits, int* bounds);
+// bounds[n] = p_vis, every inner bound a multiple of the key block, the first
+// split the longest.
+int prefix_tc_splits(int d, int p_vis, int max_splits, long spans, int sms, int* bounds);
 // maps: six tensor maps -- clean K, V; donor K, V; delta rows K, V.
 // bounds: the span splits (p.nsp + 1 values); delta_keys: keys per split of
 // the delta rows.  overlap_previous: a programmatic dependent launch of the
