@@ -2,7 +2,8 @@
 
 * ``libsplice.so``        -- the spliced decode-attention library (C ABI in
   ``include/splice.h``), from ``csrc/``.
-* ``decoder/libsplice_decoder.so`` -- the decoder's elementwise kernels.
+* ``decoder/libsplice_decoder.so`` -- the decoder's projections and
+  elementwise kernels.
 * ``synth/libsplice_synth.so`` -- the device twin of the seeded input generator.
 
 Each translation unit is compiled by its own ``nvcc`` process, in parallel,
@@ -85,11 +86,11 @@ def build(force: bool = False, verbose: bool = False) -> None:
     headers = sorted(glob.glob(os.path.join(csrc, "*.h")) + glob.glob(os.path.join(csrc, "*.cuh")) +
                      glob.glob(os.path.join(ROOT, "include", "*.h")))
     synth_src = [os.path.join(PKG, "synth", "synth.cu")]
-    decoder_src = [os.path.join(PKG, "decoder", "decoder.cu")]
+    decoder_src = sorted(glob.glob(os.path.join(PKG, "decoder", "*.cu")))
     with cf.ThreadPoolExecutor(max_workers=3) as ex:
         a = ex.submit(build_lib, "splice", sources, headers, splice_lib_path(), force, verbose)
         b = ex.submit(build_lib, "synth", synth_src, [], synth_lib_path(), force, verbose)
-        c = ex.submit(build_lib, "decoder", decoder_src, [], decoder_lib_path(), force, verbose)
+        c = ex.submit(build_lib, "decoder", decoder_src, [os.path.join(csrc, "tc_ptx.cuh"), os.path.join(PKG, "decoder", "decoder.h")], decoder_lib_path(), force, verbose)
         a.result()
         b.result()
         c.result()

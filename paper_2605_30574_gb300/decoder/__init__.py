@@ -36,7 +36,14 @@ def lib() -> ctypes.CDLL:
         L.decoder_to_bf16.argtypes = [vp, vp, l, vp]
         L.decoder_silu_mul.argtypes = [vp, vp, l, vp, l, i, vp]
         L.decoder_qkv_post.argtypes = [vp, vp, vp, vp, vp, vp, ctypes.POINTER(l), vp, vp, vp, vp, i, l, i, i, i, f, vp]
-        for fn in (L.decoder_rms_norm, L.decoder_add_rms_norm, L.decoder_add, L.decoder_to_bf16, L.decoder_silu_mul,
+        L.decoder_gemm.argtypes = [i, vp, vp, vp, vp, vp, i, i, i, vp]
+        L.decoder_gemm_plan.argtypes = [i, i, i, i, i, ctypes.POINTER(l)]
+        L.decoder_error.argtypes = [ctypes.POINTER(ctypes.c_uint)]
+        L.decoder_scratch_bytes.argtypes = [i, l, i, i, i, i]
+        L.decoder_scratch_bytes.restype = l
+        L.decoder_qkv.argtypes = [vp] * 7 + [ctypes.POINTER(l), vp, vp, vp, vp, i, l, i, i, i, i, f, vp]
+        L.decoder_block.argtypes = [vp, vp, i, vp, vp, vp, vp, vp, vp, vp, l, i, i, i, f, vp]
+        for fn in (L.decoder_qkv, L.decoder_block, L.decoder_gemm, L.decoder_gemm_plan, L.decoder_error, L.decoder_rms_norm, L.decoder_add_rms_norm, L.decoder_add, L.decoder_to_bf16, L.decoder_silu_mul,
                    L.decoder_qkv_post):
             fn.restype = i
         _LIB = L
@@ -144,3 +151,54 @@ def qkv_post(q, k, v, strides, outs, out_strides, q_norm, k_norm, inv_freq, pos,
     pointers, with (row, head) strides each."""
     _launch("decoder_qkv_post", q, k, v, *outs, (ctypes.c_long * 9)(*strides, *out_strides), q_norm.data_ptr(),
             k_norm.data_ptr(), inv_freq.data_ptr(), pos.data_ptr(), POSITIONS[pos.dtype], pos.numel(), hq, hkv, d, eps)
+
+
+# ---- a layer's halves in one call each (few rows) ----
+
+def _scratch(half, rows, D, nq, nqkv, f, device):
+    """Device scratch of a half's call, None where the shape is not one for it."""
+    n = (_LIB or lib()).decoder_scratch_bytes(half, rows, D, nq, nqkv, f)
+    return torch.empty(n, dtype=torch.uint8, device=device) if n else None
+
+
+def _aligned(*ts):
+    for t in ts:
+        if t.data_ptr() & 15:
+            return False
+    return True
+
+
+def qkv(h, in_norm, wqkv, outs, out_strides, q_norm, k_norm, inv_freq, pos, hq, hkv, d, eps) -> bool:
+    """Input norm, joined projection, per-head norm and RoPE, in one call.
+    False, and nothing done, for the shapes it does not take."""
+    rows, D = _rows(h), h.shape[-1]
+    s = _scratch(0, rows, D, hq * d, wqkv.shape[0], 0, h.device) if _aligned(wqkv) else None
+    if s is None:
+        return False
+    _launch("decoder_qkv", h.data_ptr(), in_norm.data_ptr(), wqkv.data_ptr(), s.data_ptr(), *outs,
+            (ctypes.c_long * 6)(*out_strides), q_norm.data_ptr(), k_norm.data_ptr(), inv_freq.data_ptr(),
+            pos.data_ptr(), POSITIONS[pos.dtype], rows, D, hq, hkv, d, eps)
+    return True
+
+
+def block(h, attn, wo, post_norm, w_gate, w_up, w_down, eps):
+    """What follows a layer's attention, in one call: the residual stream after
+    the layer, or None for the shapes it does not take."""
+    rows, D, nq, f = _rows(h), h.shape[-1], wo.shape[1], w_gate.shape[0]
+    s = _scratch(1, rows, D, nq, 0, f, h.device) if _aligned(attn, wo, w_gate, w_up, w_down) else None
+    if s is None:
+        return None
+    out = torch.empty_like(h)
+    _launch("decoder_block", h.data_ptr(), attn.data_ptr(), 1 if attn.dtype is BF16 else 0, wo.data_ptr(),
+            post_norm.data_ptr(), w_gate.data_ptr(), w_up.data_ptr(), w_down.data_ptr(), s.data_ptr(), out.data_ptr(),
+            rows, D, nq, f, eps)
+    return out
+
+
+def check_device_error():
+    """Raises if a bounded wait of an earlier launch on the current device ran
+    out (and clears the record); synchronises."""
+    word = ctypes.c_uint()
+    rc = lib().decoder_error(ctypes.byref(word))
+    if rc != 0 or word.value:
+        raise RuntimeError(f"decoder kernels: CUDA error {rc}, error word 0x{word.value:x}")

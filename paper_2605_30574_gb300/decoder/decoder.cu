@@ -20,10 +20,35 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "decoder.h"
+
 namespace {
 
 constexpr int kThreads = 256;
 constexpr int kKeep = 4;        // float4 of a row that a thread keeps in registers between the passes
+
+// Every kernel here is launched as a programmatic dependent of what precedes
+// it on the stream: its blocks may be set up while that still runs, wait for
+// all of it before they read or write anything, and let what follows do the
+// same.
+__device__ __forceinline__ void wait_for_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... Params, class... Args>
+int launch(void (*kernel)(Params...), dim3 grid, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return int(cudaLaunchKernelEx(&cfg, kernel, args...));
+}
 
 __device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
@@ -56,6 +81,7 @@ __global__ void __launch_bounds__(kThreads)
                     const __nv_bfloat16* __restrict__ w, float* __restrict__ h2, __nv_bfloat16* __restrict__ x, int D,
                     float eps) {
     __shared__ float part[kThreads / 32];
+    wait_for_previous();
     const size_t base = size_t(blockIdx.x) * D;
     const int t = threadIdx.x;
     float sum = 0.f;
@@ -120,6 +146,7 @@ __global__ void __launch_bounds__(kThreads)
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads)
     add_kernel(const float* h, const __nv_bfloat16* __restrict__ o, float* h2, long n) {
+    wait_for_previous();
     const long i = long(blockIdx.x) * kThreads + threadIdx.x;
     if constexpr (VEC) {
         if (i < n / 4)
@@ -134,6 +161,7 @@ __global__ void __launch_bounds__(kThreads)
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads)
     to_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ y, long n) {
+    wait_for_previous();
     const long i = long(blockIdx.x) * kThreads + threadIdx.x;
     if constexpr (VEC) {
         if (i < n / 4) {
@@ -154,6 +182,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(kThreads)
     silu_mul_kernel(const __nv_bfloat16* __restrict__ gate, const __nv_bfloat16* __restrict__ up, long ld,
                     __nv_bfloat16* __restrict__ y, int F) {
+    wait_for_previous();
     const long r = blockIdx.y;
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if constexpr (VEC) {
@@ -195,6 +224,7 @@ __global__ void __launch_bounds__(kThreads)
                     const void* __restrict__ pos, int pos_kind, int Hq, int Hkv, float eps) {
     constexpr int HALF = D / 2, V = D / 64;
     __shared__ float2 cs[HALF];
+    wait_for_previous();
     const long row = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j = blockIdx.y * (kThreads / 32) + warp;
@@ -267,72 +297,64 @@ unsigned blocks_for(long n) { return unsigned((n + kThreads - 1) / kThreads); }
 
 using bf = __nv_bfloat16;
 
+int rms_norm(const float* h, const bf* w, bf* x, long rows, int D, float eps, cudaStream_t st) {
+    const dim3 grid{unsigned(rows)};
+    const bf* none = nullptr;
+    float* no_sum = nullptr;
+    if (vec_ok(h, w, x, nullptr, D)) return launch(rms_norm_kernel<false, true>, grid, st, h, none, w, no_sum, x, D, eps);
+    return launch(rms_norm_kernel<false, false>, grid, st, h, none, w, no_sum, x, D, eps);
+}
+
+int to_bf16(const float* x, bf* y, long n, cudaStream_t st) {
+    if (vec_ok(x, y, nullptr, nullptr, n)) return launch(to_bf16_kernel<true>, dim3(blocks_for(n / 4)), st, x, y, n);
+    return launch(to_bf16_kernel<false>, dim3(blocks_for(n)), st, x, y, n);
+}
+
+size_t align256(size_t n) { return (n + 255) / 256 * 256; }
+
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
 }  // namespace
 
-// Every call returns the cudaError_t of its launch and takes contiguous rows
+// Every call returns the cudaError_t of its launches and takes contiguous rows
 // unless strides are given; rows and sizes >= 1.  rows < 2^31, n < 2^39.
 extern "C" {
 
 int decoder_rms_norm(const void* h, const void* w, void* x, long rows, int D, float eps, void* stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (vec_ok(h, w, x, nullptr, D))
-        rms_norm_kernel<false, true><<<unsigned(rows), kThreads, 0, st>>>(
-            static_cast<const float*>(h), nullptr, static_cast<const bf*>(w), nullptr, static_cast<bf*>(x), D, eps);
-    else
-        rms_norm_kernel<false, false><<<unsigned(rows), kThreads, 0, st>>>(
-            static_cast<const float*>(h), nullptr, static_cast<const bf*>(w), nullptr, static_cast<bf*>(x), D, eps);
-    return int(cudaGetLastError());
+    return rms_norm(static_cast<const float*>(h), static_cast<const bf*>(w), static_cast<bf*>(x), rows, D, eps,
+                    static_cast<cudaStream_t>(stream));
 }
 
 int decoder_add_rms_norm(const void* h, const void* o, const void* w, void* h2, void* x, long rows, int D, float eps,
                          void* stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (vec_ok(h, w, x, h2, D) && vec_ok(o, nullptr, nullptr, nullptr, D))
-        rms_norm_kernel<true, true><<<unsigned(rows), kThreads, 0, st>>>(
-            static_cast<const float*>(h), static_cast<const bf*>(o), static_cast<const bf*>(w),
-            static_cast<float*>(h2), static_cast<bf*>(x), D, eps);
-    else
-        rms_norm_kernel<true, false><<<unsigned(rows), kThreads, 0, st>>>(
-            static_cast<const float*>(h), static_cast<const bf*>(o), static_cast<const bf*>(w),
-            static_cast<float*>(h2), static_cast<bf*>(x), D, eps);
-    return int(cudaGetLastError());
+    const bool vec = vec_ok(h, w, x, h2, D) && vec_ok(o, nullptr, nullptr, nullptr, D);
+    return launch(vec ? rms_norm_kernel<true, true> : rms_norm_kernel<true, false>, dim3(unsigned(rows)),
+                  static_cast<cudaStream_t>(stream), static_cast<const float*>(h), static_cast<const bf*>(o),
+                  static_cast<const bf*>(w), static_cast<float*>(h2), static_cast<bf*>(x), D, eps);
 }
 
 int decoder_add(const void* h, const void* o, void* h2, long n, void* stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (vec_ok(h, o, h2, nullptr, n))
-        add_kernel<true><<<blocks_for(n / 4), kThreads, 0, st>>>(static_cast<const float*>(h),
-                                                                 static_cast<const bf*>(o), static_cast<float*>(h2), n);
-    else
-        add_kernel<false><<<blocks_for(n), kThreads, 0, st>>>(static_cast<const float*>(h), static_cast<const bf*>(o),
-                                                              static_cast<float*>(h2), n);
-    return int(cudaGetLastError());
+    const bool vec = vec_ok(h, o, h2, nullptr, n);
+    return launch(vec ? add_kernel<true> : add_kernel<false>, dim3(blocks_for(vec ? n / 4 : n)),
+                  static_cast<cudaStream_t>(stream), static_cast<const float*>(h), static_cast<const bf*>(o),
+                  static_cast<float*>(h2), n);
 }
 
 int decoder_to_bf16(const void* x, void* y, long n, void* stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (vec_ok(x, y, nullptr, nullptr, n))
-        to_bf16_kernel<true><<<blocks_for(n / 4), kThreads, 0, st>>>(static_cast<const float*>(x),
-                                                                     static_cast<bf*>(y), n);
-    else
-        to_bf16_kernel<false><<<blocks_for(n), kThreads, 0, st>>>(static_cast<const float*>(x), static_cast<bf*>(y), n);
-    return int(cudaGetLastError());
+    return to_bf16(static_cast<const float*>(x), static_cast<bf*>(y), n, static_cast<cudaStream_t>(stream));
 }
 
 int decoder_silu_mul(const void* gate, const void* up, long ld, void* y, long rows, int F, void* stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     // (blockIdx.y holds a row: at most 65535 rows per launch)
     for (long r0 = 0; r0 < rows; r0 += 65535) {
         const unsigned n = unsigned(rows - r0 < 65535 ? rows - r0 : 65535);
         const bf* g = static_cast<const bf*>(gate) + r0 * ld;
         const bf* u = static_cast<const bf*>(up) + r0 * ld;
         bf* out = static_cast<bf*>(y) + r0 * F;
-        if (vec_ok(g, u, out, nullptr, F) && ld % 8 == 0)
-            silu_mul_kernel<true><<<dim3(blocks_for(F / 4), n), kThreads, 0, st>>>(g, u, ld, out, F);
-        else
-            silu_mul_kernel<false><<<dim3(blocks_for(F), n), kThreads, 0, st>>>(g, u, ld, out, F);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return int(e);
+        const bool vec = vec_ok(g, u, out, nullptr, F) && ld % 8 == 0;
+        const int e = launch(vec ? silu_mul_kernel<true> : silu_mul_kernel<false>, dim3(blocks_for(vec ? F / 4 : F), n),
+                             static_cast<cudaStream_t>(stream), g, u, ld, out, F);
+        if (e != 0) return e;
     }
     return 0;
 }
@@ -342,27 +364,71 @@ int decoder_silu_mul(const void* gate, const void* up, long ld, void* y, long ro
 int decoder_qkv_post(const void* q, const void* k, const void* v, void* q_out, void* k_out, void* v_out,
                      const long* strides, const void* q_norm, const void* k_norm, const void* inv_freq,
                      const void* pos, int pos_kind, long rows, int Hq, int Hkv, int d, float eps, void* stream) {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     const HeadRows a{static_cast<const bf*>(q), strides[0], static_cast<bf*>(q_out), strides[3], strides[4]};
     const HeadRows b{static_cast<const bf*>(k), strides[1], static_cast<bf*>(k_out), strides[5], strides[6]};
     const HeadRows c{static_cast<const bf*>(v), strides[2], static_cast<bf*>(v_out), strides[7], strides[8]};
-    const bf* qn = static_cast<const bf*>(q_norm);
-    const bf* kn = static_cast<const bf*>(k_norm);
-    const float* fr = static_cast<const float*>(inv_freq);
+    auto kernel = d == 64 ? qkv_post_kernel<64> : (d == 128 ? qkv_post_kernel<128> : qkv_post_kernel<256>);
+    if (d != 64 && d != 128 && d != 256) return int(cudaErrorInvalidValue);
     const dim3 grid(unsigned(rows), unsigned((Hq + 2 * Hkv + kThreads / 32 - 1) / (kThreads / 32)));
-    switch (d) {
-        case 64:
-            qkv_post_kernel<64><<<grid, kThreads, 0, st>>>(a, b, c, qn, kn, fr, pos, pos_kind, Hq, Hkv, eps);
-            break;
-        case 128:
-            qkv_post_kernel<128><<<grid, kThreads, 0, st>>>(a, b, c, qn, kn, fr, pos, pos_kind, Hq, Hkv, eps);
-            break;
-        case 256:
-            qkv_post_kernel<256><<<grid, kThreads, 0, st>>>(a, b, c, qn, kn, fr, pos, pos_kind, Hq, Hkv, eps);
-            break;
-        default: return int(cudaErrorInvalidValue);
-    }
-    return int(cudaGetLastError());
+    return launch(kernel, grid, static_cast<cudaStream_t>(stream), a, b, c, static_cast<const bf*>(q_norm),
+                  static_cast<const bf*>(k_norm), static_cast<const float*>(inv_freq), pos, pos_kind, Hq, Hkv, eps);
+}
+
+// ---- a layer's two halves in one call each, for the rows gemm.cu takes ----
+
+// Bytes of scratch that decoder_qkv (half = 0) and decoder_block (1) need, 0
+// where the shape is not one for them.  nqkv: outputs of the joined
+// projection; nq: of q's.
+long decoder_scratch_bytes(int half, long rows, int D, int nq, int nqkv, int F) {
+    const int M = int(rows < 1 << 20 ? rows : 1 << 20);
+    if (half == 0)
+        return decoder::gemm_takes(M, nqkv, D) ? long(align256(size_t(rows) * D * 2) + size_t(rows) * nqkv * 2) : 0;
+    if (!decoder::gemm_takes(M, D, nq) || !decoder::gemm_takes(M, F, D) || !decoder::gemm_takes(M, D, F)) return 0;
+    return long(align256(size_t(rows) * nq * 2) + align256(size_t(rows) * D * 4) + align256(size_t(rows) * D * 2) +
+                size_t(rows) * F * 2);
+}
+
+// Input norm, joined projection, per-head norm and RoPE.  strides: {q row, q
+// head, k row, k head, v row, v head} of the outputs.
+int decoder_qkv(const void* h, const void* in_norm, const void* wqkv, void* scratch, void* q_out, void* k_out, void* v_out,
+                const long* strides, const void* q_norm, const void* k_norm, const void* inv_freq, const void* pos,
+                int pos_kind, long rows, int D, int Hq, int Hkv, int d, float eps, void* stream) {
+    const int nq = Hq * d, nk = Hkv * d, n = nq + 2 * nk;
+    if (!aligned16(wqkv) || !aligned16(scratch)) return int(cudaErrorInvalidValue);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    bf* x = static_cast<bf*>(scratch);
+    bf* y = reinterpret_cast<bf*>(static_cast<char*>(scratch) + align256(size_t(rows) * D * 2));
+    int e = rms_norm(static_cast<const float*>(h), static_cast<const bf*>(in_norm), x, rows, D, eps, st);
+    if (e == 0) e = decoder::gemm(decoder::kPlain, x, wqkv, nullptr, nullptr, y, int(rows), n, D, st);
+    if (e != 0) return e;
+    const long all[9] = {n, n, n, strides[0], strides[1], strides[2], strides[3], strides[4], strides[5]};
+    return decoder_qkv_post(y, y + nq, y + nq + nk, q_out, k_out, v_out, all, q_norm, k_norm, inv_freq, pos, pos_kind, rows,
+                            Hq, Hkv, d, eps, stream);
+}
+
+// Output projection and residual, norm, SwiGLU, down projection and residual.
+// attn: [rows][nq] fp32 or bf16; out: fp32 [rows][D].
+int decoder_block(const void* h, const void* attn, int attn_bf16, const void* wo, const void* post_norm, const void* w_gate,
+                  const void* w_up, const void* w_down, void* scratch, void* out, long rows, int D, int nq, int F, float eps,
+                  void* stream) {
+    for (const void* p : {attn, wo, w_gate, w_up, w_down, static_cast<const void*>(scratch)})
+        if (!aligned16(p)) return int(cudaErrorInvalidValue);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    char* at = static_cast<char*>(scratch);
+    bf* a = reinterpret_cast<bf*>(at);
+    at += align256(size_t(rows) * nq * 2);
+    float* h2 = reinterpret_cast<float*>(at);
+    at += align256(size_t(rows) * D * 4);
+    bf* x = reinterpret_cast<bf*>(at);
+    at += align256(size_t(rows) * D * 2);
+    bf* y = reinterpret_cast<bf*>(at);
+    const int M = int(rows);
+    int e = attn_bf16 ? 0 : to_bf16(static_cast<const float*>(attn), a, rows * nq, st);
+    if (e == 0) e = decoder::gemm(decoder::kResid, attn_bf16 ? attn : a, wo, nullptr, h, h2, M, D, nq, st);
+    if (e == 0) e = rms_norm(h2, static_cast<const bf*>(post_norm), x, rows, D, eps, st);
+    if (e == 0) e = decoder::gemm(decoder::kSwiglu, x, w_gate, w_up, nullptr, y, M, F, D, st);
+    if (e == 0) e = decoder::gemm(decoder::kResid, y, w_down, nullptr, h2, out, M, D, F, st);
+    return e;
 }
 
 }  // extern "C"

@@ -1,0 +1,15 @@
+// Internal declarations of the decoder library.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace decoder {
+
+constexpr int kPlain = 0, kResid = 1, kSwiglu = 2;
+
+// The fused projections of gemm.cu (see decoder_gemm) and the shapes they take.
+bool gemm_takes(int M, int N, int K);
+int gemm(int mode, const void* x, const void* w0, const void* w1, const void* h, void* y, int M, int N, int K,
+         cudaStream_t stream);
+
+}  // namespace decoder

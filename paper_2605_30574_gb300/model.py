@@ -82,15 +82,21 @@ class RandomDecoder:
         g.manual_seed(seed)
         bf = dict(dtype=torch.bfloat16, device=self.device)
 
+        def normal(*shape, scale=std):
+            return torch.randn(*shape, generator=g, dtype=torch.float32, device=self.device) * scale
+
         def rnd(*shape, scale=std):
-            return (torch.randn(*shape, generator=g, dtype=torch.float32, device=self.device) * scale).to(torch.bfloat16)
+            return normal(*shape, scale=scale).to(torch.bfloat16)
 
         def rows(*heights):
             # matrices that read the same input, as consecutive rows of one:
             # one GEMM gives all their outputs
-            m = torch.cat([rnd(n, dims.d_model) for n in heights])
-            ends = [sum(heights[:i + 1]) for i in range(len(heights))]
-            return [m[e - n:e] for n, e in zip(heights, ends)]
+            m, out = torch.empty((sum(heights), dims.d_model), **bf), []
+            for n in heights:
+                at = sum(w.shape[0] for w in out)
+                out.append(m[at:at + n])
+                out[-1].copy_(normal(n, dims.d_model))
+            return out
 
         D, Hq, Hkv, d, F = dims.d_model, dims.num_q_heads, dims.num_kv_heads, dims.head_dim, dims.ffn
         self.embed = rnd(dims.vocab, D, scale=1.0)
@@ -124,7 +130,7 @@ class RandomDecoder:
         if self._kernels(l, h, pos):
             q, k, v = (torch.empty((*h.shape[:-1], n, dims.head_dim), dtype=torch.bfloat16, device=h.device)
                        for n in (dims.num_q_heads, dims.num_kv_heads, dims.num_kv_heads))
-            self._qkv_into(l, K.rms_norm(h, w["in_norm"], dims.rms_eps), pos, q, k, v)
+            self._qkv_into(l, h, pos, q, k, v)
             return q, k, v
         x = _rms_norm(h, w["in_norm"], dims.rms_eps).to(torch.bfloat16)
         q = (x @ w["wq"].t()).unflatten(-1, (dims.num_q_heads, dims.head_dim))
@@ -138,8 +144,7 @@ class RandomDecoder:
         """Residual stream after layer l given its attention output attn [..., Hq, d]."""
         dims, w = self.dims, self.layers[l]
         if self._kernels(l, h) and self._attn_ok(h, attn):
-            h, o = self._block(l, h, attn)
-            return K.add_(h, o)
+            return self._block(l, h, attn)
         h = h + (attn.to(torch.bfloat16).flatten(-2) @ w["wo"].t()).float()
         x = _rms_norm(h, w["post_norm"], dims.rms_eps).to(torch.bfloat16)
         gate = x @ w["w_gate"].t()
@@ -192,13 +197,18 @@ class RandomDecoder:
         return (k.dtype is v.dtype is torch.bfloat16 and k.shape == v.shape == shape and K.plain((k, v), ())
                 and k.device == h.device and k.data_ptr() % 16 == v.data_ptr() % 16 == 0)
 
-    def _qkv_into(self, l: int, x: torch.Tensor, pos: torch.Tensor, q, k, v) -> None:
-        """q, k, v of layer l from its normed input rows x, written to the
-        given bf16 tensors [..., n, H, d] (q, v as they are; any strides whose
-        rows of d elements are contiguous)."""
+    def _qkv_into(self, l: int, h: torch.Tensor, pos: torch.Tensor, q, k, v) -> None:
+        """q, k, v of layer l from the residual stream h, written to the given
+        bf16 tensors [..., n, H, d] (any strides whose rows of d elements are
+        contiguous)."""
         dims, w = self.dims, self.layers[l]
         d, nq, nk = dims.head_dim, dims.num_q_heads * dims.head_dim, dims.num_kv_heads * dims.head_dim
+        outs, strides = [t.data_ptr() for t in (q, k, v)], [s for t in (q, k, v) for s in t.stride()[-3:-1]]
+        head = (w["q_norm"], w["k_norm"], self.inv_freq, pos, dims.num_q_heads, dims.num_kv_heads, d, dims.rms_eps)
         wqkv = K.joined(w["wq"], w["wk"], w["wv"])
+        if wqkv is not None and K.qkv(h, w["in_norm"], wqkv, outs, strides, *head):
+            return
+        x = K.rms_norm(h, w["in_norm"], dims.rms_eps)
         if wqkv is not None:
             y = torch.nn.functional.linear(x, wqkv)
             p, ld = y.data_ptr(), (nq + 2 * nk,) * 3
@@ -206,15 +216,15 @@ class RandomDecoder:
         else:
             y = [torch.nn.functional.linear(x, w[n]) for n in ("wq", "wk", "wv")]
             src, ld = [t.data_ptr() for t in y], (nq, nk, nk)
-        K.qkv_post(*src, ld, [t.data_ptr() for t in (q, k, v)], [s for t in (q, k, v) for s in t.stride()[-3:-1]],
-                   w["q_norm"], w["k_norm"], self.inv_freq, pos, dims.num_q_heads, dims.num_kv_heads, d,
-                   dims.rms_eps)
+        K.qkv_post(*src, ld, outs, strides, *head)
 
-    def _block(self, l: int, h: torch.Tensor, attn: torch.Tensor):
-        """Layer l after its attention: the residual stream before the MLP's
-        output is added (a tensor of its own), and that output (bf16)."""
+    def _block(self, l: int, h: torch.Tensor, attn: torch.Tensor) -> torch.Tensor:
+        """block_out through the kernels."""
         dims, w = self.dims, self.layers[l]
         linear = torch.nn.functional.linear
+        out = K.block(h, attn, w["wo"], w["post_norm"], w["w_gate"], w["w_up"], w["w_down"], dims.rms_eps)
+        if out is not None:
+            return out
         a = attn if attn.dtype is torch.bfloat16 else K.to_bf16(attn)
         h, x = K.add_rms_norm(h, linear(a.flatten(-2), w["wo"]), w["post_norm"], dims.rms_eps)
         w_gu = K.joined(w["w_gate"], w["w_up"])
@@ -222,7 +232,7 @@ class RandomDecoder:
             y = K.silu_mul_joined(linear(x, w_gu))
         else:
             y = K.silu_mul(linear(x, w["w_gate"]), linear(x, w["w_up"]))
-        return h, linear(y, w["w_down"])
+        return K.add_(h, linear(y, w["w_down"]))
 
     # -- prefill ----------------------------------------------------------
     @torch.no_grad()
@@ -239,8 +249,7 @@ class RandomDecoder:
             if type(self).qkv is RandomDecoder.qkv and self._kernels(l, h, pos) and self._store_ok(h, kl, vl):
                 # straight into the stores
                 q = torch.empty((h.shape[0], dims.num_q_heads, dims.head_dim), dtype=torch.bfloat16, device=h.device)
-                self._qkv_into(l, K.rms_norm(h, self.layers[l]["in_norm"], dims.rms_eps), pos, q, kl.transpose(0, 1),
-                               vl.transpose(0, 1))
+                self._qkv_into(l, h, pos, q, kl.transpose(0, 1), vl.transpose(0, 1))
                 kh, vh = kl[None], vl[None]
             else:
                 q, k, v = self.qkv(l, h, pos)               # [T_p, H, d]
@@ -354,6 +363,7 @@ class SpliceDecode:
                 y = torch.where(done, torch.full_like(y, eos), y)
             toks.append(y)
         S.splice_check_device_error(self.desc)
+        K.check_device_error()
         return torch.stack(toks, dim=1)
 
     def close(self):

@@ -159,3 +159,70 @@ def test_prefill_into_stores_and_into_copies(hq, hkv, d, T):
     want = model.prefill(tokens, kf, vf)
     got = model.prefill(tokens, k, v)
     assert torch.equal(k.float(), kf) and torch.equal(v.float(), vf) and torch.equal(got, want)
+
+
+def gemm(mode, x, w0, w1=None, h=None):
+    M, k, N = x.shape[0], x.shape[1], w0.shape[0]
+    y = torch.full((M + 1, N), float("nan"), dtype=torch.float32 if mode == 1 else torch.bfloat16, device="cuda")
+    p = [t.data_ptr() if t is not None else None for t in (x, w0, w1, h, y)]
+    assert K.lib().decoder_gemm(mode, *p, M, N, k, torch.cuda.current_stream().cuda_stream) == 0
+    K.check_device_error()
+    assert bool(y[M].isnan().all())             # nothing past the last row
+    return y[:M].double()
+
+
+# one CTA per tile and clusters of up to eight; ragged rows, features and K
+@pytest.mark.parametrize("M", [1, 15, 16, 17, 64, 100, 128, 129, 400])
+@pytest.mark.parametrize("N,k", [(1, 8), (130, 72), (640, 1000), (4096, 512), (2000, 4096), (20000, 136), (256, 12288)])
+def test_fused_projections(M, N, k):
+    """fp32 sums of K exact products, each addition of 16 of them truncated at
+    2^-23 of the largest partial sum at most; then the output's own rounding."""
+    g = gen(M + N + k)
+    x, wa, wb = (randn(g, n, k, dtype=torch.bfloat16) for n in (M, N, N))
+    wa, wb = ((w.float() * k ** -0.5).bfloat16() for w in (wa, wb))
+    h = randn(g, M, N)
+    a, b = (x.double() @ w.double().t() for w in (wa, wb))
+    ma, mb = (x.double().abs() @ w.double().abs().t() for w in (wa, wb))
+    e = (k / 16 + 12) * 2.0 ** -23
+    assert bool(((gemm(0, x, wa) - a).abs() <= e * ma + 2.0 ** -8 * a.abs() + 1e-30).all())
+    assert bool(((gemm(1, x, wa, h=h) - (h.double() + a)).abs() <= e * ma + 2.0 ** -23 * (h.double() + a).abs()).all())
+    s = torch.nn.functional.silu(a) * b
+    # (|silu'| <= 1.1)
+    bound = 1.1 * e * ma * (b.abs() + e * mb) + e * mb * a.abs() + (2.0 ** -8 + 2.0 ** -20) * s.abs() + 1e-30
+    assert bool(((gemm(2, x, wa, wb) - s).abs() <= bound).all())
+
+
+def test_fused_projection_rows_are_independent():
+    """An infinity or NaN in a row of x stays in that row, the same bits with
+    or without it; the same call twice gives the same bits."""
+    g = gen(3)
+    x, w = randn(g, 20, 1024, dtype=torch.bfloat16), randn(g, 300, 1024, dtype=torch.bfloat16)
+    want = gemm(0, x, w)
+    assert torch.equal(gemm(0, x, w), want)
+    x[7, 100], x[12, 0] = float("inf"), float("nan")
+    got = gemm(0, x, w)
+    rest = [r for r in range(20) if r not in (7, 12)]
+    assert torch.equal(got[rest], want[rest])
+    assert not bool(got[7].isfinite().any()) and bool(got[12].isnan().all())
+
+
+# one row; the last rows of one tile, the first of a second; a third of a tile
+# more; rows that the library takes in the second half only, and in both
+@pytest.mark.parametrize("rows,ffn", [(1, 1544), (128, 1544), (129, 1544), (300, 1544), (300, 12288), (4500, 12288)])
+def test_layer_on_either_side_of_the_row_limit(rows, ffn):
+    """A half of the layer is one call on the fused projections or the
+    library's GEMMs with kernels between; both meet the torch expressions."""
+    model = RandomDecoder(DecoderDims(1, 6, 2, 128, 1024, ffn, 40), seed=4)
+    g = gen(rows)
+    assert (K.lib().decoder_scratch_bytes(0, rows, 1024, 768, 1280, 0) > 0) == (rows < 4500)
+    assert (K.lib().decoder_scratch_bytes(1, rows, 1024, 768, 0, ffn) > 0) == (ffn < 2000)
+    h, pos, attn = randn(g, rows, 1024), torch.arange(rows, device="cuda"), randn(g, rows, 6, 128)
+    (q, k, v), (qt, kt, vt) = both(model, h, pos)
+    for a, b in ((q, qt), (k, kt), (v, vt)):
+        close(a, b, scale=2 * b.abs().amax(-1, keepdim=True).expand_as(b))
+    want = model.block_out(0, h.clone().requires_grad_(), attn).detach()
+    kept = h.clone()
+    got = model.block_out(0, h, attn)
+    assert torch.equal(h, kept) and got.data_ptr() != h.data_ptr()
+    assert (got - want).abs().max() <= 4 * ULP * (want - h).abs().max()
+    K.check_device_error()
