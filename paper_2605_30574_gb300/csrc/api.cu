@@ -173,6 +173,10 @@ splice_status create_common(const splice_model_shape* sh, int P, int Tp, int Dsl
     return SPLICE_OK;
 }
 
+// The rate at which a long generated-span pass streams, and the share of its
+// time that a prompt-span pass beside it may take.
+constexpr double kGenBytesPerUs = 6.2e6, kPrefixShare = 0.6;
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // (Re)builds the device table block of a descriptor from its host plan and
@@ -478,6 +482,28 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
                                  gs_keys * splice::kPrefixFirstGenRatio < prefix_keys)));
     p.gs_after_prefix = gs_work && prefix_launched && prefix_first && !d->profiling ? 1 : 0;
     p.prefix_after_gs = gs_work && prefix_launched && !prefix_first && !d->profiling ? 1 : 0;
+    // A short prompt-span pass ahead of a long generated-span pass leaves it
+    // SMs from the start: the generated-span pass streams at the memory's rate
+    // from half of them, while the prompt-span pass, a chain of latencies, uses
+    // little of it.  As few CTAs as end within kPrefixShare of the
+    // generated-span pass's time (and before its warps have more items to
+    // merge later than they keep).  Measured at 152, 96, 76 and 56 CTAs: eight
+    // rows per kv head, 300 cells, 79.7, 75.4, 74.9, 74.7 us; Qwen3-4B-shaped
+    // 118.0, 116.4, 115.7, 115.1; where the prompt spans hold more, it costs
+    // (252 cells of 2255 keys: 69.8, 102.1), and where the generated-span pass
+    // is short of warps itself (seven rows of 256 dims: 141.7, 141.9, 149).
+    if (p.gs_after_prefix && splice::generated_span_streams_from_half(sh.head_dim, p.G)) {
+        const double gs_us = double(gs_keys) * sh.head_dim * 4 / kGenBytesPerUs;
+        const double per_warp = double(d->B) * sh.num_kv_heads * p.nss /
+                                splice::generated_span_resident_warps(sh.head_dim, p.G);
+        const double most_us = gs_us * std::min(kPrefixShare, (splice::kMaxPending - 1) / std::max(per_warp, 1.0));
+        for (int part = 6; part <= 16; part += 2) {
+            const int ctas = std::max(1, d->sms * part / 19);
+            if (splice::prefix_tc_us(sh.head_dim, prefix_items, tc_keys, ctas) > most_us) continue;
+            p.prefix_ctas = ctas;
+            break;
+        }
+    }
     // Behind the prompt-span pass, with one prompt-span and one
     // generated-span split per row and no delta rows, the generated-span
     // pass merges every row itself and writes the output: ZERO rows at the

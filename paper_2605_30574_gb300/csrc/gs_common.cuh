@@ -62,7 +62,7 @@ __device__ __forceinline__ float merge_two(bool has_span, float w_span, float o_
 
 // Items a warp may leave unmerged until its end (with P.gs_merge): those
 // that end before the prompt-span pass has completed.
-constexpr int kPend = 8;
+constexpr int kPend = kMaxPending;
 
 // n / d for 0 <= n < 2^31 by a multiply and a shift, for a divisor fixed
 // per launch (Granlund and Montgomery, "Division by invariant integers using

@@ -1001,7 +1001,8 @@ int launch_d(const TcParams& tp, const CUtensorMap* m, cudaStream_t st, bool ove
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
-    const unsigned grid = unsigned(tp.n_items < sms ? tp.n_items : sms);
+    const int most = tp.a.prefix_ctas > 0 && tp.a.prefix_ctas < sms ? tp.a.prefix_ctas : sms;
+    const unsigned grid = unsigned(tp.n_items < most ? tp.n_items : most);
     if (!overlap_previous) {
         prefix_tc_kernel<D, SHORT><<<grid, kThreads, C::SMEM, st>>>(m[0], m[1], m[2], m[3], m[4], m[5], tp);
         return 0;
@@ -1097,6 +1098,12 @@ int prefix_tc_splits(int d, int p_vis, int max_splits, long spans, int sms, int*
         bounds[i + 1] = b < p_vis ? b : p_vis;
     }
     return ns;
+}
+
+double prefix_tc_us(int d, long items, int keys, int ctas) {
+    const int bn = prefix_tc_box_rows(d);
+    const double item = (keys + bn - 1) / bn * (d == 256 ? kBlockUs256 : kBlockUs) + kItemUs;
+    return double((items + ctas - 1) / ctas) * item;
 }
 
 int launch_prefix_tc(const AttnParams& p, const void* maps, const int* bounds, int delta_keys, void* stream,

@@ -754,6 +754,8 @@ bool generated_span_can_merge(int d, int G) {
     return fma_kernel(d, G) ? G * d <= 512 : gs::mma_can_merge(d, G);   // GT * F <= 16 in gs_kernel, F = d / 32
 }
 
+bool generated_span_streams_from_half(int d, int G) { return d < 256 || fma_kernel(d, G); }
+
 int launch_generated_span(const AttnParams& p, void* stream, bool overlap_previous) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long n_items = long(p.B) * p.Hkv * p.nss;

@@ -41,6 +41,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "gs_common.cuh"
@@ -750,8 +751,8 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
                     item_of(P, dv, pend[k], it);
                     const size_t row0 = size_t(it.s) * P.Hq + it.h * P.G;
                     const size_t gen0 = size_t(kMaxPrefixSplits) * P.B * P.Hq + row0;
-                    // (the loads of four passes go out before any is used)
-                    constexpr int K = C::NP < 4 ? C::NP : 4;
+                    // (the loads of all passes go out before any is used)
+                    constexpr int K = C::NP;
                     for (int r0 = e_row; r0 - e_row < P.G; r0 += K * C::RPP) {
                         float2 ml_gen[K], ml_span[K];
                         float4 og[K][2], os[K][2];
@@ -819,7 +820,9 @@ int launch_mma_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
-    const Shape<D, NT> sh(p.G);
+    Shape<D, NT> sh(p.G);
+    // few items: spread over the SMs rather than a CTA's warps
+    sh.warps = int(std::min<long>(sh.warps, (long(n_items) + sms - 1) / sms));
     const long want = (long(n_items) + sh.warps - 1) / sh.warps;
     const long cap = long(sh.ctas) * sms;
     cudaLaunchConfig_t cfg = {};

@@ -18,6 +18,9 @@ namespace splice {
 constexpr int kMaxPrefixSplits = 8;
 constexpr int kMaxSuffixSplits = 8;
 constexpr int kMaxSplits = kMaxPrefixSplits + kMaxSuffixSplits;
+// Generated-span items that a warp may leave unmerged until its end, when the
+// generated-span pass merges.
+constexpr int kMaxPending = 8;
 // Rows of one tensor-core prefix tile (tcgen05 M).
 constexpr int kTileRows = 128;
 // Prompt-span splits: a span's first split holds kPrefixFirstSplitKeys keys,
@@ -135,6 +138,7 @@ struct AttnParams {
     int fuse_append;              // the generated-span pass also appends entry step - 1 (see kn, vn)
     int gs_after_prefix;          // the generated-span pass runs behind the prompt-span pass of the call
     int prefix_after_gs;          // the prompt-span pass runs behind the generated-span pass of the call
+    int prefix_ctas;              // CTAs of the prompt-span pass at the most (0: one per multiprocessor)
     int gs_merge;                 // the generated-span pass merges rows itself (see launch_generated_span)
     int p_chunk, s_chunk;         // keys per split
     int n_tiles;
@@ -165,6 +169,9 @@ int generated_span_resident_warps(int d, int G);
 // Whether the generated-span pass is built with its merge path for head
 // dim d and GQA group G (AttnParams::gs_merge may be set only then).
 bool generated_span_can_merge(int d, int G);
+// Whether half of the multiprocessors run the generated-span pass at the
+// memory's rate.
+bool generated_span_streams_from_half(int d, int G);
 // overlap_previous: the launch directly follows the last pass of the same
 // call on the stream (programmatic dependent launch; the kernel waits for it,
 // and that pass's completion implies the other pass's).
@@ -187,6 +194,8 @@ int prefix_tc_box_rows(int d);
 // bounds[n] = p_vis, every inner bound a multiple of the key block, the first
 // split the longest.
 int prefix_tc_splits(int d, int p_vis, int max_splits, long spans, int sms, int* bounds);
+// Estimated time of `items` items of up to `keys` keys on `ctas` CTAs, in us.
+double prefix_tc_us(int d, long items, int keys, int ctas);
 // maps: six tensor maps -- clean K, V; donor K, V; delta rows K, V.
 // bounds: the span splits (p.nsp + 1 values); delta_keys: keys per split of
 // the delta rows.  overlap_previous: a programmatic dependent launch of the
