@@ -50,17 +50,18 @@ using decoder::kPlain;
 using decoder::kResid;
 using decoder::kSwiglu;
 
-constexpr int kFeat = 128, kBK = 64, kOutWarps = 8, kThreads = 64 + 32 * kOutWarps, kMaxStages = 8, kMaxSplit = 8, kCtasPerSm = 2;
+constexpr int kFeat = 128, kBK = 64, kOutWarps = 8, kThreads = 64 + 32 * kOutWarps, kMaxStages = 8, kMaxSplit = 8;
 constexpr uint32_t kWBytes = kFeat * kBK * 2;    // 128 rows of W, one K block
 constexpr uint32_t kChunkBytes = 16 * kFeat * 4;  // 16 rows' sums of a tile
-constexpr int kSmemMax = 112 * 1024;             // two CTAs per SM
+constexpr int kSmemMax = 226 * 1024;
 constexpr unsigned kErrLoad = 1, kErrMma = 2, kErrOut = 4, kErrDrain = 8;
 
 __device__ unsigned g_error;
 
 struct GemmParams {
     int M, N, K;
-    int mp;                 // rows of x per CTA, the MMA's columns: M rounded up to 16, 128 at the most
+    int mp;                 // rows of x per CTA, the MMA's columns: a multiple of 16, 256 at the most
+    int ctas_per_sm;        // 2 up to 128 rows, else 1
     int tiles_m;            // of mp rows
     int kblocks, split;     // K blocks; CTAs that share them
     int stages;
@@ -70,7 +71,9 @@ struct GemmParams {
     void* y;
 };
 
-__device__ __forceinline__ float silu(float g) { return g / (1.f + expf(-g)); }
+// (a few units of 2^-24 off, far inside the output's bf16 rounding; the exact
+// division and expf cost a tile of 144 rows 3.4 us of its epilogue warps)
+__device__ __forceinline__ float silu(float g) { return __fdividef(g, 1.f + __expf(-g)); }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
@@ -107,7 +110,7 @@ __device__ __forceinline__ void store16(const GemmParams& P, int m, int feature,
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm)
+__global__ void __launch_bounds__(kThreads, 2)
     gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w0,
                 const __grid_constant__ CUtensorMap tm_w1, const GemmParams P) {
     constexpr int PARTS = MODE == kSwiglu ? 2 : 1;     // W matrices, accumulators
@@ -316,26 +319,50 @@ bool make_map(CUtensorMap* m, const void* base, int rows, int K, int box_rows) {
                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The launch's shape (host arithmetic only).
-void plan(int mode, GemmParams& p, int sms) {
+// Ring and split of tiles of p.mp rows (host arithmetic only).
+void plan_tiles(int mode, GemmParams& p, int sms) {
     const int parts = mode == kSwiglu ? 2 : 1;
-    p.tiles = (p.N + kFeat - 1) / kFeat;
-    p.mp = std::min(128, (p.M + 15) / 16 * 16);
     p.tiles_m = (p.M + p.mp - 1) / p.mp;
-    p.kblocks = (p.K + kBK - 1) / kBK;
+    p.ctas_per_sm = p.mp <= 128 ? 2 : 1;
     p.stage_bytes = parts * kWBytes + uint32_t(p.mp) * kBK * 2;
-    p.stages = std::min(kMaxStages, int((kSmemMax - 1024) / p.stage_bytes));
+    p.stages = std::min(kMaxStages, int((kSmemMax / p.ctas_per_sm - 1024) / p.stage_bytes));
     p.tmem_cols = 32;
     while (p.tmem_cols < uint32_t(p.mp * parts)) p.tmem_cols *= 2;
     // CTAs per tile: as many as are resident together (clusters do not pack
     // the SMs whole, hence the eighth left over), each with two K blocks
     // at least, and few enough that the ring holds the sums they trade.
-    const int room = kCtasPerSm * sms * 7 / 8;
+    const int room = p.ctas_per_sm * sms * 7 / 8;
     p.split = std::max(1, std::min(std::min(kMaxSplit, int(room / (long(p.tiles) * p.tiles_m))), p.K / (2 * kBK)));
     const int chunks = p.mp / 16;
     while (p.split > 1 && uint32_t(p.split * ((chunks + p.split - 1) / p.split) * parts) * kChunkBytes >
                               uint32_t(p.stages) * p.stage_bytes)
         --p.split;
+}
+
+// The launch's shape (host arithmetic only).  Up to 128 rows one tile of rows
+// (W streams from HBM once).  More rows are bound by the MMAs, a tile of 256
+// rows and a K block of 64 taking 640 clocks: even tiles of 128 to 256 rows,
+// of the least time in whole waves (512 rows, gate and up of 12288: 96 tiles
+// of features by two of rows are 1.26 waves of 256 rows, by three 1.9 of 176).
+void plan(int mode, GemmParams& p, int sms) {
+    p.tiles = (p.N + kFeat - 1) / kFeat;
+    p.kblocks = (p.K + kBK - 1) / kBK;
+    GemmParams best = p;
+    double least = 0;
+    for (int tm = (p.M + 255) / 256; tm <= (p.M + 127) / 128; ++tm) {
+        GemmParams c = p;
+        c.mp = ((p.M + tm - 1) / tm + 15) / 16 * 16;
+        plan_tiles(mode, c, sms);
+        const long ctas = long(c.tiles) * c.tiles_m * c.split, at_once = long(c.ctas_per_sm) * sms;
+        const double block = (mode == kSwiglu ? 2 : 1) * 2.5 * c.mp + 130.0;
+        const double clocks = double((ctas + at_once - 1) / at_once) *
+                                  (c.ctas_per_sm * block * c.kblocks / c.split + 6000.0) + (c.split > 1 ? 5000.0 : 0.0);
+        if (least == 0 || clocks < least) {
+            least = clocks;
+            best = c;
+        }
+    }
+    p = best;
 }
 
 template <int MODE>
@@ -376,11 +403,9 @@ int launch(const void* x, const void* w0, const void* w1, GemmParams p, cudaStre
 namespace decoder {
 
 bool gemm_takes(int M, int N, int K) {
-    // TMA rows are multiples of 16 bytes.  More than 128 rows read W once more
-    // (from L2) per 128: while that takes no longer than the 20 us that a
-    // library GEMM takes of the host.
+    // TMA rows are multiples of 16 bytes.
     if (M < 1 || M > 65536 || N < 1 || K < 8 || K % 8 != 0) return false;
-    return M <= 128 || (M + 127L) / 128 * N * K * 2 <= 64L << 20;
+    return M <= kGemmRows || (M + 255L) / 256 * N * K * 2 <= 64L << 20;
 }
 
 int gemm(int mode, const void* x, const void* w0, const void* w1, const void* h, void* y, int M, int N, int K,
