@@ -431,14 +431,17 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
         if (tc_keys > 0) p.nsd = std::min(max_splits, (d->delta_max + tc_keys - 1) / tc_keys);
     }
     {
-        // Generated-span items: (sequence, kv head, key split).  Split so
+        // Generated-span items: (sequence, kv head, row chunk, key split).  Split so
         // every resident warp gets about two items, but keep at least 64 keys
         // per split.  Every split costs a partial state to write and merge;
         // the prompt-span pass queued behind this one fills the SMs its last
         // warps leave idle, so few splits pay off even where the items do not
         // share out evenly over the warps.
-        const long base_items = long(d->B) * sh.num_kv_heads;
-        const long want = 2L * splice::generated_span_resident_warps(sh.head_dim, p.G);
+        const long pairs = long(d->B) * sh.num_kv_heads;
+        p.gs_rows = splice::generated_span_rows(sh.head_dim, p.G, pairs);
+        p.gs_chunks = (p.G + p.gs_rows - 1) / p.gs_rows;
+        const long base_items = pairs * p.gs_chunks;
+        const long want = 2L * splice::generated_span_resident_warps(sh.head_dim, p.gs_rows);
         int ns = int(std::min<long>(splice::kMaxSuffixSplits, std::max<long>(1, (want + base_items - 1) / base_items)));
         ns = std::min(ns, std::max(1, s_vis / 64));
         p.nss = s_vis > 0 ? ns : 0;
@@ -492,10 +495,10 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
     // 118.0, 116.4, 115.7, 115.1; where the prompt spans hold more, it costs
     // (252 cells of 2255 keys: 69.8, 102.1), and where the generated-span pass
     // is short of warps itself (seven rows of 256 dims: 141.7, 141.9, 149).
-    if (p.gs_after_prefix && splice::generated_span_streams_from_half(sh.head_dim, p.G)) {
+    if (p.gs_after_prefix && splice::generated_span_streams_from_half(sh.head_dim, p.gs_rows)) {
         const double gs_us = double(gs_keys) * sh.head_dim * 4 / kGenBytesPerUs;
-        const double per_warp = double(d->B) * sh.num_kv_heads * p.nss /
-                                splice::generated_span_resident_warps(sh.head_dim, p.G);
+        const double per_warp = double(d->B) * sh.num_kv_heads * p.gs_chunks * p.nss /
+                                splice::generated_span_resident_warps(sh.head_dim, p.gs_rows);
         const double most_us = gs_us * std::min(kPrefixShare, (splice::kMaxPending - 1) / std::max(per_warp, 1.0));
         for (int part = 6; part <= 16; part += 2) {
             const int ctas = std::max(1, d->sms * part / 19);
@@ -511,7 +514,7 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
     // (a flag it reads without waiting), else at the warp's end after the
     // grid dependency wait.  No merge kernel is launched then.
     p.gs_merge = p.gs_after_prefix && p.nss == 1 && p.nsp == 1 && !p.delta_on &&
-                         splice::generated_span_can_merge(sh.head_dim, p.G)
+                         splice::generated_span_can_merge(sh.head_dim, p.gs_rows)
                      ? 1
                      : 0;
     auto launch_prefix = [&]() -> splice_status {

@@ -79,21 +79,24 @@ struct FastDiv {
 };
 
 struct ItemDivs {
-    FastDiv nss, hkv;
+    FastDiv nss, chunks, hkv;
 };
 
 // One work item: where its rows and keys are.  The issue cursor decodes
 // each item once and hands it to the consumer through the warp's ring
 // (eight ints, idx -1 for the end of the walk).
 struct Item {
-    int idx, s, h, split, k0, k1, nblk;
+    int idx, s, h, split, k0, k1, nblk, rc;
 };
 
-// Work item idx = (sequence * Hkv + kv head) * splits + key split.
+// Work item idx = ((sequence * Hkv + kv head) * row chunks + row chunk) *
+// splits + key split.
 __device__ __forceinline__ void item_of(const AttnParams& P, const ItemDivs& dv, int idx, Item& it) {
     it.idx = idx;
-    const int sh = dv.nss.div(idx);
-    it.split = idx - sh * P.nss;
+    const int rem = dv.nss.div(idx);
+    it.split = idx - rem * P.nss;
+    const int sh = dv.chunks.div(rem);
+    it.rc = rem - sh * P.gs_chunks;
     it.s = dv.hkv.div(sh);
     it.h = sh - it.s * P.Hkv;
     it.k0 = P.s_lo + it.split * P.s_chunk;
@@ -112,9 +115,9 @@ __device__ __forceinline__ size_t span_base(const AttnParams& P, int s, int h) {
 // the number of multiprocessors.
 int launch_mma(const AttnParams& p, cudaStream_t stream, bool overlap_previous);
 // Warps of the tensor-core kernel that an SM holds, and whether it is built
-// with its merge path.
-int mma_warps_per_sm(int d, int G);
-bool mma_can_merge(int d, int G);
+// with its merge path, at `rows` query rows per item.
+int mma_warps_per_sm(int d, int rows);
+bool mma_can_merge(int d, int rows);
 
 }  // namespace gs
 }  // namespace splice

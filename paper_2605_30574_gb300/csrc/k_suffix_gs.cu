@@ -1,12 +1,12 @@
-// Generated-span pass on CUDA cores, for one query row per kv head (and two or
-// four of 256 dims; k_suffix_mma.cu has the rest and the rule is at the end
+// Generated-span pass on CUDA cores, for items of one query row (and two or
+// four of 256 dims; k_suffix_mma.cu has the rest and the rules are at the end
 // of this file): attention of the G query rows of one (sequence, kv head) over
 // that sequence's own generated-span K/V (§3: the decode step attends over the
 // prompt span and the t generated entries).
 //
 // HBM-bound streaming kernel:
-//   * persistent warps walking work items (sequence, kv head, key split) and,
-//     inside an item, blocks of 16 keys: a fixed stream per warp when this
+//   * persistent warps walking work items (sequence, kv head, row chunk, key
+//     split) and, inside an item, blocks of 16 keys: a fixed stream per warp when this
 //     pass goes first, items claimed at run time (one ahead) when
 //     it runs behind the prompt-span pass, so warps that start late (on SMs
 //     that pass still holds) simply take fewer; the issue cursor decodes
@@ -206,14 +206,14 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
     // item it takes, decoded (then the end, idx -1), for the consumer.  It
     // runs two blocks ahead and every item has a block (the host keeps at
     // least 64 keys per split), so it is at most two items ahead ----
-    const ItemDivs dv{FastDiv(P.nss), FastDiv(P.Hkv)};
+    const ItemDivs dv{FastDiv(P.nss), FastDiv(P.gs_chunks), FastDiv(P.Hkv)};
     Item iss;
     int iss_idx = first_item < n_items ? first_item : -1, iss_b = 0, recorded = 0;
     bool iss_ok = false;
     auto record = [&](const Item& e) {
         if (lane == 0) {
             ring[2 * (recorded & 3)] = make_int4(e.idx, e.s, e.h, e.split);
-            ring[2 * (recorded & 3) + 1] = make_int4(e.k0, e.k1, e.nblk, 0);
+            ring[2 * (recorded & 3) + 1] = make_int4(e.k0, e.k1, e.nblk, e.rc);
         }
         ++recorded;
     };
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             tc::mbar_arrive_expect_tx(bar0 + 8 * stg, 2 * bytes + (first ? C::QROWS : 0u));
             if (first)
                 bulk_copy_plain(wbase + C::OFF_Q + (iss_items & 1) * C::QROWS,
-                                P.q + (size_t(iss.s) * P.Hq + iss.h * GT) * D, C::QROWS, bar0 + 8 * stg);
+                                P.q + (size_t(iss.s) * P.Hq + iss.h * P.G + iss.rc * GT) * D, C::QROWS, bar0 + 8 * stg);
             if (bytes) {
                 bulk_copy(dst, P.ks + iss_base + size_t(j) * D, bytes, bar0 + 8 * stg, pol);
                 bulk_copy(dst + C::BK * C::ROW, P.vs + iss_base + size_t(j) * D, bytes, bar0 + 8 * stg, pol);
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
         const int4 e0 = ring[2 * (taken & 3)];
         if (e0.x < 0) break;
         const int4 e1 = ring[2 * (taken & 3) + 1];
-        const Item it{e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z};
+        const Item it{e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
         // merges in this pass: the rows' source (a ZERO row needs no
         // prompt-span state) and, until it has been seen set, the prompt-span
         // pass's completion flag, read now and used at the item's end
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             const int jb = it.k0 + b * 16;
             if (tail && b == it.nblk - 1) {
                 // the step's own entry: its row of the stage from registers,
-                // and into the store
+                // and (once per (sequence, kv head)) into the store
                 const int rj = P.s_hi - 1 - jb;
                 const size_t ent = ((size_t(it.s) * P.N + P.layer) * P.Hkv + it.h) * size_t(P.T) + (P.s_hi - 1);
 #pragma unroll
@@ -378,7 +378,8 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
                         const bool isk = c < D / 8;
                         const int cc = isk ? c : c - D / 8;
                         *reinterpret_cast<uint4*>((isk ? kst : vst) + rj * C::ROW + cc * 16) = nkv[i];
-                        reinterpret_cast<uint4*>(isk ? P.ks_w : P.vs_w)[ent * (D / 8) + cc] = nkv[i];
+                        if (it.rc == 0)
+                            reinterpret_cast<uint4*>(isk ? P.ks_w : P.vs_w)[ent * (D / 8) + cc] = nkv[i];
                     }
                 }
                 __syncwarp();
@@ -529,7 +530,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             if (merge_here && has_span) {
 #pragma unroll
                 for (int g = 0; g < GT; ++g) {
-                    const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;   // split 0's slot
+                    const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;   // split 0's slot
                     ml_span[g] = __ldcg(P.ws_ml + row);
                     const float* sp = P.ws_o + row * D + dim0;
                     if constexpr (F == 2) {
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             const bool zero_span = !has_span && P.p_hi > P.p_lo;
 #pragma unroll
             for (int g = 0; g < GT; ++g) {
-                const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;
+                const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;
                 // the row's (m, l) as lane 0 would store it: the lanes' row
                 // sums can differ in the last bit (each lane adds its pair's
                 // two terms in its own order)
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
             const int slot = kMaxPrefixSplits + it.split;
 #pragma unroll
             for (int g = 0; g < GT; ++g) {
-                const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;
+                const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;
                 const size_t idx2 = size_t(slot) * P.B * P.Hq + row;
                 float* op = P.ws_o + idx2 * D + dim0;
                 if constexpr (F == 2) {
@@ -670,7 +671,7 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
                     item_of(P, dv, pend[k], it);
 #pragma unroll
                     for (int g = 0; g < GT; ++g) {
-                        const size_t row = size_t(it.s) * P.Hq + it.h * GT + g;
+                        const size_t row = size_t(it.s) * P.Hq + it.h * P.G + it.rc * GT + g;
                         const size_t gen = size_t(kMaxPrefixSplits) * P.B * P.Hq + row;
                         const float2 ml_gen = __ldcg(P.ws_ml + gen), ml_span = __ldcg(P.ws_ml + row);
                         float og[F], os[F];
@@ -730,7 +731,7 @@ int launch_gs_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap_
 
 }  // namespace
 
-// The FMA kernel above for one query row per kv head (d = 64, 128, 256) and
+// The FMA kernel above for items of one query row (d = 64, 128, 256) and
 // for two or four of 256 dims; the tensor-core kernel for the rest.  At one
 // row the FMA kernel has less to do per key (140 x 8 heads of 128 dims x 500
 // keys: 44.7 us against 45.6); rows of 256 dims leave the tensor-core kernel
@@ -742,26 +743,44 @@ int launch_gs_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap_
 // against 168; eight rows, 300 x 8 heads x 277 keys: 110 against 58).
 static bool fma_kernel(int d, int G) { return G == 1 || (d == 256 && (G == 2 || G == 4)); }
 
-int generated_span_resident_warps(int d, int G) {
+int generated_span_rows(int d, int G, long pairs) {
+    // With few pairs a warp's own latency is all that there is to wait for:
+    // then items of fewer rows run side by side (and read K and V once each,
+    // mostly from L2).  The line is one item per warp.  At 256 dims they take
+    // the FMA kernel, by the largest of four, two and one that divides G
+    // (three rows, 56 pairs: 12.8 us against 14.5); past eight rows of fewer
+    // dims, eight at a time (sixteen rows, 152 pairs: 16.3 against 19).
+    if (G <= 8 && (d < 256 || fma_kernel(d, G))) return G;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (d == 256) {
+        const int few = G % 4 == 0 ? 4 : (G % 2 == 0 ? 2 : 1);
+        return pairs * (G / few) <= 6L * sms ? few : G;
+    }
+    return pairs <= long(sms) * gs::mma_warps_per_sm(d, G) ? 8 : G;
+}
+
+int generated_span_resident_warps(int d, int rows) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // FMA kernel: two 4-warp CTAs per SM (d <= 128), three 2-warp CTAs per SM (d = 256)
-    return sms * (fma_kernel(d, G) ? (d == 256 ? 6 : 8) : gs::mma_warps_per_sm(d, G));
+    return sms * (fma_kernel(d, rows) ? (d == 256 ? 6 : 8) : gs::mma_warps_per_sm(d, rows));
 }
 
-bool generated_span_can_merge(int d, int G) {
-    return fma_kernel(d, G) ? G * d <= 512 : gs::mma_can_merge(d, G);   // GT * F <= 16 in gs_kernel, F = d / 32
+bool generated_span_can_merge(int d, int rows) {
+    return fma_kernel(d, rows) ? rows * d <= 512 : gs::mma_can_merge(d, rows);   // GT * F <= 16 in gs_kernel, F = d / 32
 }
 
-bool generated_span_streams_from_half(int d, int G) { return d < 256 || fma_kernel(d, G); }
+bool generated_span_streams_from_half(int d, int rows) { return d < 256 || fma_kernel(d, rows); }
 
 int launch_generated_span(const AttnParams& p, void* stream, bool overlap_previous) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const long n_items = long(p.B) * p.Hkv * p.nss;
+    const long n_items = long(p.B) * p.Hkv * p.gs_chunks * p.nss;
     if (n_items == 0) return 0;
-    if (!fma_kernel(p.D, p.G)) return gs::launch_mma(p, st, overlap_previous);
-    switch (p.D * 8 + p.G) {
+    if (!fma_kernel(p.D, p.gs_rows)) return gs::launch_mma(p, st, overlap_previous);
+    switch (p.D * 8 + p.gs_rows) {
         case 64 * 8 + 1: return launch_gs_t<64, 1>(p, int(n_items), st, overlap_previous);
         case 128 * 8 + 1: return launch_gs_t<128, 1>(p, int(n_items), st, overlap_previous);
         case 256 * 8 + 1: return launch_gs_t<256, 1>(p, int(n_items), st, overlap_previous);

@@ -3,7 +3,8 @@
 // attends over the prompt span and the t generated entries).
 //
 // HBM-bound streaming kernel:
-//   * persistent warps walking work items (sequence, kv head, key split) and,
+//   * persistent warps walking work items (sequence, kv head, row chunk, key
+//     split; one chunk but for more than eight rows in a small launch) and,
 //     inside an item, blocks of 16 keys: a fixed stream per warp when this
 //     pass goes first, items claimed at run time (one ahead) when it runs
 //     behind the prompt-span pass, so warps that start late (on SMs that pass
@@ -176,9 +177,9 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
-    uint8_t* ws = smem + warp * C::per_warp(P.G);
+    uint8_t* ws = smem + warp * C::per_warp(P.gs_rows);
     const uint32_t wbase = tc::smem_u32(ws);
-    float* stg = reinterpret_cast<float*>(ws + C::off_stg(P.G));
+    float* stg = reinterpret_cast<float*>(ws + C::off_stg(P.gs_rows));
     int4* ring = reinterpret_cast<int4*>(ws + C::OFF_TAKEN);
     int* pend = reinterpret_cast<int*>(ws + C::OFF_PEND);
     int npend = 0;
@@ -249,14 +250,14 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
     // item it takes, decoded (then the end, idx -1), for the consumer.  It
     // runs two blocks ahead and every item has a block (the host makes no
     // empty split), so it is at most two items ahead ----
-    const ItemDivs dv{FastDiv(P.nss), FastDiv(P.Hkv)};
+    const ItemDivs dv{FastDiv(P.nss), FastDiv(P.gs_chunks), FastDiv(P.Hkv)};
     Item iss;
     int iss_idx = first_item < n_items ? first_item : -1, iss_b = 0, recorded = 0;
     bool iss_ok = false;
     auto record = [&](const Item& e) {
         if (lane == 0) {
             ring[2 * (recorded & 3)] = make_int4(e.idx, e.s, e.h, e.split);
-            ring[2 * (recorded & 3) + 1] = make_int4(e.k0, e.k1, e.nblk, 0);
+            ring[2 * (recorded & 3) + 1] = make_int4(e.k0, e.k1, e.nblk, e.rc);
         }
         ++recorded;
     };
@@ -287,9 +288,10 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
             // an item's first block also brings the item's query rows
             // (contiguous in q) into its query buffer
             if (iss_b == 0) {
-                const uint32_t qd = wbase + C::OFF_Q + (iss_items & 1) * (P.G * C::ROW);
-                const uint16_t* qs = P.q + (size_t(iss.s) * P.Hq + iss.h * P.G) * D;
-                for (int e = lane; e < P.G * C::CH; e += 32) {
+                const uint32_t qd = wbase + C::OFF_Q + (iss_items & 1) * (P.gs_rows * C::ROW);
+                const uint16_t* qs = P.q + (size_t(iss.s) * P.Hq + iss.h * P.G + iss.rc * P.gs_rows) * D;
+                const int rows = min(P.gs_rows, P.G - iss.rc * P.gs_rows);
+                for (int e = lane; e < rows * C::CH; e += 32) {
                     const int r = e / C::CH, c = e % C::CH;
                     cp16_plain(qd + r * C::ROW + ((c ^ (r & 7)) * 16), qs + e * 8);
                 }
@@ -342,13 +344,6 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
     const int v_row = (lane & 7) + (lane >> 4) * 8, v_ch = (lane >> 3) & 1;     // V (transposed)
     const int q_ch = lane >> 3;                                                 // Q: four chunks of eight rows
     const uint32_t k_at = k_row * C::ROW + ((k_ch ^ (k_row & 7)) * 16), v_at = v_row * C::ROW + ((v_ch ^ (v_row & 7)) * 16);
-    // (row tiles past G read the last row again: their columns are not used)
-    uint32_t q_at[NT];
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-        const int r = min(8 * n + (lane & 7), P.G - 1);
-        q_at[n] = r * C::ROW + ((q_ch ^ (r & 7)) * 16);
-    }
     // chunk 2 c + (0, 1) of a swizzled row, given the row's chunk 0 (or 1)
     auto chunk2 = [](uint32_t at, int c) { return (at ^ ((c & 3) * 32)) + (c >> 2) * 128; };
     // the epilogue's lanes: row e_row of a pass, 16 bytes e_c
@@ -358,7 +353,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
         const int4 e0 = ring[2 * (taken & 3)];
         if (e0.x < 0) break;
         const int4 e1 = ring[2 * (taken & 3) + 1];
-        const Item it{e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z};
+        const Item it{e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
         // merges in this pass: the rows' source (a ZERO row needs no
         // prompt-span state) and, until it has been seen set, the prompt-span
         // pass's completion flag, read now and used at the item's end
@@ -384,7 +379,15 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
                                        : reinterpret_cast<const uint4*>(P.vn)[rowc + c - D / 8];
             }
         }
-        const uint32_t qaddr = wbase + C::OFF_Q + (cons_items & 1) * (P.G * C::ROW);
+        const uint32_t qaddr = wbase + C::OFF_Q + (cons_items & 1) * (P.gs_rows * C::ROW);
+        // (columns past the item's rows read its last row again and are not used)
+        const int rows = min(P.gs_rows, P.G - it.rc * P.gs_rows);
+        uint32_t q_at[NT];
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            const int r = min(8 * n + (lane & 7), rows - 1);
+            q_at[n] = r * C::ROW + ((q_ch ^ (r & 7)) * 16);
+        }
         if (it.nblk > 0) ++cons_items;
         // Q as the column operand: fragment kk covers dims 16 kk .. 16 kk + 15
         uint32_t qf[C::QREG ? NT : 1][C::QREG ? D / 16 : 1][2];
@@ -426,7 +429,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
             }
             if (tail && b == it.nblk - 1) {
                 // the step's own entry: its row of the stage from registers,
-                // and into the store
+                // and (once per (sequence, kv head)) into the store
                 const int rj = P.s_hi - 1 - jb;
                 const size_t ent = ((size_t(it.s) * P.N + P.layer) * P.Hkv + it.h) * size_t(P.T) + (P.s_hi - 1);
 #pragma unroll
@@ -437,7 +440,8 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
                         const int cc = isk ? c : c - D / 8;
                         *reinterpret_cast<uint4*>(ws + stg_i * C::STAGE + (isk ? 0u : C::KBYTES) + rj * C::ROW +
                                                   ((cc ^ (rj & 7)) * 16)) = nkv[i];
-                        reinterpret_cast<uint4*>(isk ? P.ks_w : P.vs_w)[ent * (D / 8) + cc] = nkv[i];
+                        if (it.rc == 0)
+                            reinterpret_cast<uint4*>(isk ? P.ks_w : P.vs_w)[ent * (D / 8) + cc] = nkv[i];
                     }
                 }
                 __syncwarp();
@@ -577,7 +581,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
         // them; past that the warp waits for the prompt-span grid here) ----
         bool merge_here = false;
         const bool has_span = code != SPLICE_SRC_ZERO;
-        const size_t row0 = size_t(it.s) * P.Hq + it.h * P.G;
+        const size_t row0 = size_t(it.s) * P.Hq + it.h * P.G + it.rc * P.gs_rows;
         constexpr int NPM = C::MERGE ? C::NP : 1;
         float2 ml_span[NPM];
         float4 o_span[C::AHEAD][NPM];
@@ -601,7 +605,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
 #pragma unroll
                 for (int k = 0; k < NPM; ++k) {
                     const int r = k * C::RPP + e_row;
-                    if (r < P.G) {
+                    if (r < rows) {
                         ml_span[k] = __ldcg(P.ws_ml + row0 + r);     // split 0's slot
                         const float4* sp = reinterpret_cast<const float4*>(P.ws_o + (row0 + r) * D) + e_c;
 #pragma unroll
@@ -649,7 +653,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
                     for (int e = 0; e < 2; ++e) {
                         const int r = 8 * n + 2 * t4 + e;
                         float z = 0.f;
-                        if (r < P.G) {
+                        if (r < rows) {
                             const uint16_t* qr = P.q + (row0 + r) * D;
 #pragma unroll 1
                             for (int c = 0; c < D; ++c)
@@ -673,7 +677,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
         float mr[C::NP], lr[C::NP], w_span[NPM], w_gen[NPM], inv[NPM];
 #pragma unroll
         for (int k = 0; k < C::NP; ++k) {
-            if (k * C::RPP >= P.G) break;
+            if (k * C::RPP >= rows) break;
             const int r = k * C::RPP + e_row, src = (r & 7) >> 1;
             float mm = 0.f, ll = 0.f;
 #pragma unroll
@@ -700,7 +704,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
 #pragma unroll
                 for (int k = 0; k < NPM; ++k) {
                     const int r = k * C::RPP + e_row;
-                    if (r < P.G) o_span[0][k] = __ldcg(reinterpret_cast<const float4*>(P.ws_o + (row0 + r) * D) + C::LPR + e_c);
+                    if (r < rows) o_span[0][k] = __ldcg(reinterpret_cast<const float4*>(P.ws_o + (row0 + r) * D) + C::LPR + e_c);
                 }
             }
             __syncwarp();
@@ -710,13 +714,13 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
                 for (int i = 0; i < D / 32; ++i)
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
-                        if (8 * n + 2 * t4 + (e & 1) < P.G)
+                        if (8 * n + 2 * t4 + (e & 1) < rows)
                             stg[(8 * n + 2 * t4 + (e & 1)) * C::LDO + 16 * i + g8 + (e >> 1) * 8] = o[n][hh * (D / 32) + i][e];
             __syncwarp();
 #pragma unroll
             for (int k = 0; k < C::NP; ++k) {
                 const int r = k * C::RPP + e_row;
-                if (r < P.G) {
+                if (r < rows) {
                     const float4 x = *reinterpret_cast<const float4*>(stg + r * C::LDO + 4 * e_c);
                     if (C::MERGE && merge_here) {
                         const float4 sp = has_span ? o_span[hh % C::AHEAD][k % NPM] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -749,17 +753,18 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
                 for (int k = 0; k < npend; ++k) {
                     Item it;
                     item_of(P, dv, pend[k], it);
-                    const size_t row0 = size_t(it.s) * P.Hq + it.h * P.G;
+                    const size_t row0 = size_t(it.s) * P.Hq + it.h * P.G + it.rc * P.gs_rows;
+                    const int rows = min(P.gs_rows, P.G - it.rc * P.gs_rows);
                     const size_t gen0 = size_t(kMaxPrefixSplits) * P.B * P.Hq + row0;
                     // (the loads of all passes go out before any is used)
                     constexpr int K = C::NP;
-                    for (int r0 = e_row; r0 - e_row < P.G; r0 += K * C::RPP) {
+                    for (int r0 = e_row; r0 - e_row < rows; r0 += K * C::RPP) {
                         float2 ml_gen[K], ml_span[K];
                         float4 og[K][2], os[K][2];
 #pragma unroll
                         for (int i = 0; i < K; ++i) {
                             const int r = r0 + i * C::RPP;
-                            if (r < P.G) {
+                            if (r < rows) {
                                 ml_gen[i] = __ldcg(P.ws_ml + gen0 + r);
                                 ml_span[i] = __ldcg(P.ws_ml + row0 + r);
 #pragma unroll
@@ -772,7 +777,7 @@ __global__ void __launch_bounds__(GM<D, NT>::MAX_WARPS * 32, GM<D, NT>::REG_WARP
 #pragma unroll
                         for (int i = 0; i < K; ++i) {
                             const int r = r0 + i * C::RPP;
-                            if (r < P.G) {
+                            if (r < rows) {
                                 float w_span, w_gen;
                                 const float inv = merge_two_weights(true, ml_span[i], ml_gen[i].x, ml_gen[i].y, false, 0,
                                                                     &w_span, &w_gen);
@@ -820,7 +825,7 @@ int launch_mma_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
-    Shape<D, NT> sh(p.G);
+    Shape<D, NT> sh(p.gs_rows);
     // few items: spread over the SMs rather than a CTA's warps
     sh.warps = int(std::min<long>(sh.warps, (long(n_items) + sms - 1) / sms));
     const long want = (long(n_items) + sh.warps - 1) / sh.warps;
@@ -828,7 +833,7 @@ int launch_mma_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(want < cap ? want : cap));
     cfg.blockDim = dim3(unsigned(sh.warps) * 32);
-    cfg.dynamicSmemBytes = sh.warps * C::per_warp(p.G);
+    cfg.dynamicSmemBytes = sh.warps * C::per_warp(p.gs_rows);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -841,8 +846,8 @@ int launch_mma_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap
 }  // namespace
 
 int launch_mma(const AttnParams& p, cudaStream_t stream, bool overlap_previous) {
-    const int n_items = int(long(p.B) * p.Hkv * p.nss);
-    const bool two = p.G > 8;
+    const int n_items = int(long(p.B) * p.Hkv * p.gs_chunks * p.nss);
+    const bool two = p.gs_rows > 8;
     switch (p.D) {
         case 64:
             return two ? launch_mma_t<64, 2>(p, n_items, stream, overlap_previous)
@@ -859,18 +864,18 @@ int launch_mma(const AttnParams& p, cudaStream_t stream, bool overlap_previous) 
 
 namespace {
 template <int D, int NT>
-int warps_per_sm(int G) {
-    const Shape<D, NT> s(G);
+int warps_per_sm(int rows) {
+    const Shape<D, NT> s(rows);
     return s.warps * s.ctas;
 }
 }  // namespace
 
-int mma_warps_per_sm(int d, int G) {
-    if (G > 8) return d == 64 ? warps_per_sm<64, 2>(G) : (d == 128 ? warps_per_sm<128, 2>(G) : warps_per_sm<256, 2>(G));
-    return d == 64 ? warps_per_sm<64, 1>(G) : (d == 128 ? warps_per_sm<128, 1>(G) : warps_per_sm<256, 1>(G));
+int mma_warps_per_sm(int d, int rows) {
+    if (rows > 8) return d == 64 ? warps_per_sm<64, 2>(rows) : (d == 128 ? warps_per_sm<128, 2>(rows) : warps_per_sm<256, 2>(rows));
+    return d == 64 ? warps_per_sm<64, 1>(rows) : (d == 128 ? warps_per_sm<128, 1>(rows) : warps_per_sm<256, 1>(rows));
 }
 
-bool mma_can_merge(int d, int G) { return d * (G > 8 ? 2 : 1) <= 256; }   // GM::MERGE
+bool mma_can_merge(int d, int rows) { return d * (rows > 8 ? 2 : 1) <= 256; }   // GM::MERGE
 
 }  // namespace gs
 }  // namespace splice

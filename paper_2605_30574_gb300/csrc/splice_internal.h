@@ -139,6 +139,7 @@ struct AttnParams {
     int gs_after_prefix;          // the generated-span pass runs behind the prompt-span pass of the call
     int prefix_after_gs;          // the prompt-span pass runs behind the generated-span pass of the call
     int prefix_ctas;              // CTAs of the prompt-span pass at the most (0: one per multiprocessor)
+    int gs_rows, gs_chunks;       // query rows of a generated-span item, items that share a kv head's rows
     int gs_merge;                 // the generated-span pass merges rows itself (see launch_generated_span)
     int p_chunk, s_chunk;         // keys per split
     int n_tiles;
@@ -165,13 +166,17 @@ int launch_append(const uint16_t* kn, const uint16_t* vn, uint16_t* ks, uint16_t
 // flag (sched[4]) and fenced, waits for it only before it exits, and lets
 // its own dependents launch only once its work is done.
 int launch_generated_span(const AttnParams& p, void* stream, bool overlap_previous);
-int generated_span_resident_warps(int d, int G);
+// Query rows of one item, for `pairs` (sequence, kv head) pairs: all G, or
+// fewer where the pairs are few.
+int generated_span_rows(int d, int G, long pairs);
+// The functions below take the rows of an item.
+int generated_span_resident_warps(int d, int rows);
 // Whether the generated-span pass is built with its merge path for head
-// dim d and GQA group G (AttnParams::gs_merge may be set only then).
-bool generated_span_can_merge(int d, int G);
+// dim d (AttnParams::gs_merge may be set only then).
+bool generated_span_can_merge(int d, int rows);
 // Whether half of the multiprocessors run the generated-span pass at the
 // memory's rate.
-bool generated_span_streams_from_half(int d, int G);
+bool generated_span_streams_from_half(int d, int rows);
 // overlap_previous: the launch directly follows the last pass of the same
 // call on the stream (programmatic dependent launch; the kernel waits for it,
 // and that pass's completion implies the other pass's).

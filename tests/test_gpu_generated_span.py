@@ -62,7 +62,7 @@ class Span:
 def test_every_group_size(G, d):
     # one entry; a block short of one, whole, and one over; several splits,
     # the last ragged; more items than warps
-    for t, cells in ((1, 3), (15, 2), (16, 2), (17, 2), (64, 1), (209, 3), (530, 2), (33, 700)):
+    for t, cells in ((1, 3), (15, 2), (16, 2), (17, 2), (64, 1), (209, 3), (530, 2), (33, 700), (5, 1000)):
         s = Span(G, d, t, cells, seed=t)
         want, bound = s.exact()
         err = (s.step().double() - want).abs()
