@@ -37,7 +37,7 @@ def lib() -> ctypes.CDLL:
         L.decoder_silu_mul.argtypes = [vp, vp, l, vp, l, i, vp]
         L.decoder_qkv_post.argtypes = [vp, vp, vp, vp, vp, vp, ctypes.POINTER(l), vp, vp, vp, vp, i, l, i, i, i, f, vp]
         L.decoder_gemm.argtypes = [i, vp, vp, vp, vp, vp, i, i, i, vp]
-        L.decoder_gemm_plan.argtypes = [i, i, i, i, i, ctypes.POINTER(l)]
+        L.decoder_gemm_plan.argtypes = [i, i, i, i, ctypes.POINTER(i), ctypes.POINTER(l)]
         L.decoder_error.argtypes = [ctypes.POINTER(ctypes.c_uint)]
         L.decoder_scratch_bytes.argtypes = [i, l, i, i, i, i]
         L.decoder_scratch_bytes.restype = l
@@ -153,7 +153,7 @@ def qkv_post(q, k, v, strides, outs, out_strides, q_norm, k_norm, inv_freq, pos,
             k_norm.data_ptr(), inv_freq.data_ptr(), pos.data_ptr(), POSITIONS[pos.dtype], pos.numel(), hq, hkv, d, eps)
 
 
-# ---- a layer's halves in one call each (few rows) ----
+# ---- a layer's halves in one call each ----
 
 def _scratch(half, rows, D, nq, nqkv, f, device):
     """Device scratch of a half's call, None where the shape is not one for it."""

@@ -374,7 +374,7 @@ int decoder_qkv_post(const void* q, const void* k, const void* v, void* q_out, v
                   static_cast<const bf*>(k_norm), static_cast<const float*>(inv_freq), pos, pos_kind, Hq, Hkv, eps);
 }
 
-// ---- a layer's two halves in one call each, for the rows gemm.cu takes ----
+// ---- a layer's two halves in one call each, for the shapes gemm.cu takes ----
 
 // Bytes of scratch that decoder_qkv (half = 0) and decoder_block (1) need, 0
 // where the shape is not one for them.  nqkv: outputs of the joined

@@ -6,7 +6,6 @@
 namespace decoder {
 
 constexpr int kPlain = 0, kResid = 1, kSwiglu = 2;
-constexpr int kGemmRows = 512;
 
 // The fused projections of gemm.cu (see decoder_gemm) and the shapes they take.
 bool gemm_takes(int M, int N, int K);
