@@ -651,14 +651,18 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
         tc::mbar_wait(bar0 + 8 * (consumed & 1), uint32_t(consumed >> 1) & 1u, &no_abort, P.err, kErrWaitGsDrain,
                       10000000000ull);
     }
-    if (P.gs_after_prefix) {
+    if (P.gs_after_prefix && (blockIdx.x == 0 || npend > 0)) {
         // Behind the prompt-span pass: this grid's completion must imply that
         // pass's, so the merge queued behind this grid sees both (with
-        // P.gs_merge no merge is queued: this grid writes every output).
+        // P.gs_merge no merge is queued: this grid writes every output).  One
+        // CTA that waits for that pass is enough; the others go, and leave
+        // their SMs to this grid's CTAs that found none beside that pass (36 x
+        // 8 heads, sixteen rows of 256 dims, three keys each beside 48
+        // prompt-span CTAs: FIGURES).
         // Then the work behind may launch (the merge waits for this whole
         // grid before it reads anything); every CTA of this grid is running
-        // by the time all of them have signalled, so those CTAs never hold
-        // an SM it still needs.
+        // by the time all of them have signalled or gone, so those CTAs never
+        // hold an SM it still needs.
         asm volatile("griddepcontrol.wait;" ::: "memory");
         // The items left unmerged: the prompt-span states are complete and
         // visible now; this warp's own partial states are re-read (the same
