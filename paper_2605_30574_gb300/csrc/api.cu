@@ -513,10 +513,27 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
     // item's end, the others there once the prompt-span pass has completed
     // (a flag it reads without waiting), else at the warp's end after the
     // grid dependency wait.  No merge kernel is launched then.
-    p.gs_merge = p.gs_after_prefix && p.nss == 1 && p.nsp == 1 && !p.delta_on &&
-                         splice::generated_span_can_merge(sh.head_dim, p.gs_rows)
-                     ? 1
-                     : 0;
+    // Unless the generated-span pass ends well before the prompt-span pass
+    // with more than an item per warp: then hardly any item could be merged at
+    // its end, a few per warp one after the other at the very end, and the
+    // merge kernel does them side by side (104 x 8 heads, eight rows of 256
+    // dims, seven keys each, prompts of 1713: 51.2 us against 46.5; 1000 x 2
+    // heads, four rows of 128, 60 keys: 32.3 against 27.4).  Short of that,
+    // merging at the items' ends saves the states' way through memory (1000 x
+    // 8 heads, eight rows of 128, 7 keys, prompts of 300: 62 us against 67).
+    // An item takes a warp 2 us and 0.25 a row, or its bytes' time.
+    bool merges = p.gs_after_prefix && p.nss == 1 && p.nsp == 1 && !p.delta_on &&
+                  splice::generated_span_can_merge(sh.head_dim, p.gs_rows);
+    if (merges) {
+        const double items = double(d->B) * sh.num_kv_heads * p.gs_chunks;
+        const double warps = double(splice::generated_span_resident_warps(sh.head_dim, p.gs_rows)) *
+                             (prefix_items < d->sms ? double(d->sms - prefix_items) / d->sms : 1.0);
+        const double gs_us = std::max(double(gs_keys) * sh.head_dim * 4 / kGenBytesPerUs,
+                                      std::ceil(items / warps) * (2 + 0.25 * p.gs_rows) * std::min(sh.head_dim, 128) / 128);
+        if (items > 0.9 * warps && 1.2 * gs_us < splice::prefix_tc_us(sh.head_dim, prefix_items, tc_keys, d->sms))
+            merges = false;
+    }
+    p.gs_merge = merges ? 1 : 0;
     auto launch_prefix = [&]() -> splice_status {
         // Tensor maps over the stores viewed as [rows][d]; the delta rows
         // have the donor store's layout.

@@ -91,3 +91,32 @@ def test_windows_shorter_than_the_span():
         ref = np.stack([oracle.decode_attn(wl, inp, s, seqs[s], 1, step) for s in which])
         assert_close(a.run(1, step)[which].cpu().numpy(), ref, f"t={step}")
     S.splice_check_device_error(a.desc)
+
+
+# eight and three rows on the tensor-core kernel, one on the FMA kernel; a step
+# whose generated spans are short beside the prompts' and the first whole block
+@pytest.mark.parametrize("d,hq,hkv,cells", [(256, 16, 2, 420), (128, 12, 4, 500), (64, 4, 4, 1400)])
+def test_short_generated_spans_beside_long_prompts(d, hq, hkv, cells):
+    """The prompt-span pass goes first, and the merge kernel merges (three
+    launches and the same bits as with the passes the other way round)."""
+    wl = workload(2100, d, hq, hkv, 4, 16)
+    seqs = (wl.sequences() * (cells // len(wl.sequences()) + 1))[:cells]
+    b = SweepBatch(wl, seqs=seqs)
+    inp = CachedInputs(wl)
+    for l, t in ((0, 3), (1, 16)):
+        b.gen_inputs(l, t)
+        outs = []
+        for order in (1, 2):
+            S.splice_debug_pass_order(b.desc, order)
+            b.out.fill_(float("nan"))
+            before = S.splice_kernel_launches(b.desc)
+            b.step(l, t)
+            torch.cuda.synchronize()
+            assert S.splice_kernel_launches(b.desc) - before == 3
+            outs.append(b.out.clone())
+        S.splice_debug_pass_order(b.desc, 0)
+        assert torch.equal(*outs), (l, t)
+        which = [0, cells // 2, cells - 1]
+        ref = np.stack([oracle.decode_attn(wl, inp, s, seqs[s], l, t) for s in which])
+        assert_close(outs[0][which].cpu().numpy(), ref, f"d={d} l={l} t={t}")
+    S.splice_check_device_error(b.desc)
