@@ -195,6 +195,23 @@ def block(h, attn, wo, post_norm, w_gate, w_up, w_down, eps):
     return out
 
 
+# Up to this many rows the fused projections stream a large weight matrix faster
+# than the library (151936 x 4096, fp32 out: 1 row 178 us against 205, 256 rows
+# 224 against 237); with more, and two tiles of rows, they do not (320 rows 271
+# against 257, 400 rows 320 against 298).
+LOGITS_ROWS = 256
+
+
+def logits(x, w):
+    """x w^T in fp32, or None for the shapes it does not take."""
+    rows, D = _rows(x), x.shape[-1]
+    if rows > LOGITS_ROWS or D % 8 or w.shape[0] == 0 or not _aligned(x, w):
+        return None
+    y = torch.empty((*x.shape[:-1], w.shape[0]), dtype=torch.float32, device=x.device)
+    _launch("decoder_gemm", 1, x.data_ptr(), w.data_ptr(), None, None, y.data_ptr(), rows, w.shape[0], D)
+    return y
+
+
 def check_device_error():
     """Raises if a bounded wait of an earlier launch on the current device ran
     out (and clears the record); synchronises."""

@@ -1,7 +1,8 @@
 // The decoder's projections on tcgen05, with what follows them fused in:
 //
 //   PLAIN   y  = bf16(x W^T)                      q, k, v in one
-//   RESID   h2 = h + x W^T        (fp32)          attention output, MLP output
+//   RESID   h2 = h + x W^T        (fp32)          attention output, MLP output;
+//                                                 without h, logits
 //   SWIGLU  y  = bf16(silu(x Wg^T) * (x Wu^T))    gate and up in one
 //
 // x [M][K], W [N][K] bf16, both K-major; sums in fp32, rounded to bf16 only
@@ -550,7 +551,7 @@ int gemm(int mode, const void* x, const void* w0, const void* w1, const void* h,
 
 extern "C" {
 
-// mode 0: y bf16 [M][N] = x w0^T; 1: y fp32 [M][N] = h + x w0^T; 2: y bf16
+// mode 0: y bf16 [M][N] = x w0^T; 1: y fp32 [M][N] = h + x w0^T (h NULL: 0); 2: y bf16
 // [M][N] = silu(x w0^T) * (x w1^T).  All contiguous, 16-byte aligned; shapes
 // that gemm_takes.  Returns a cudaError_t.
 int decoder_gemm(int mode, const void* x, const void* w0, const void* w1, const void* h, void* y, int M, int N, int K,

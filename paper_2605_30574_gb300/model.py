@@ -156,6 +156,9 @@ class RandomDecoder:
                 and K.plain((h,), (self.final_norm, self.lm_head))):
             x = K.rms_norm(h, self.final_norm, self.dims.rms_eps)
             # (the product's fp32 sums as they are, in one pass over the logits)
+            y = K.logits(x, self.lm_head)
+            if y is not None:
+                return y
             return torch.mm(x.flatten(0, -2) if x.dim() > 1 else x[None], self.lm_head.t(),
                             out_dtype=torch.float32).view(*h.shape[:-1], -1)
         x = _rms_norm(h, self.final_norm, self.dims.rms_eps).to(torch.bfloat16)

@@ -187,6 +187,7 @@ def test_fused_projections(M, N, k):
     e = (k / 16 + 12) * 2.0 ** -23
     assert bool(((gemm(0, x, wa) - a).abs() <= e * ma + 2.0 ** -8 * a.abs() + 1e-30).all())
     assert bool(((gemm(1, x, wa, h=h) - (h.double() + a)).abs() <= e * ma + 2.0 ** -23 * (h.double() + a).abs()).all())
+    assert bool(((gemm(1, x, wa) - a).abs() <= e * ma + 2.0 ** -23 * a.abs()).all())
     s = torch.nn.functional.silu(a) * b
     # (|silu'| <= 1.1)
     bound = 1.1 * e * ma * (b.abs() + e * mb) + e * mb * a.abs() + (2.0 ** -8 + 2.0 ** -20) * s.abs() + 1e-30
