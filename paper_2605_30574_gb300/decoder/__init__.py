@@ -43,7 +43,8 @@ def lib() -> ctypes.CDLL:
         L.decoder_scratch_bytes.restype = l
         L.decoder_qkv.argtypes = [vp] * 7 + [ctypes.POINTER(l), vp, vp, vp, vp, i, l, i, i, i, i, f, vp]
         L.decoder_block.argtypes = [vp, vp, i, vp, vp, vp, vp, vp, vp, vp, l, i, i, i, f, vp]
-        for fn in (L.decoder_qkv, L.decoder_block, L.decoder_gemm, L.decoder_gemm_plan, L.decoder_error, L.decoder_rms_norm, L.decoder_add_rms_norm, L.decoder_add, L.decoder_to_bf16, L.decoder_silu_mul,
+        L.decoder_causal.argtypes = [vp] * 4 + [l, i, i, i, f, vp]
+        for fn in (L.decoder_qkv, L.decoder_block, L.decoder_causal, L.decoder_gemm, L.decoder_gemm_plan, L.decoder_error, L.decoder_rms_norm, L.decoder_add_rms_norm, L.decoder_add, L.decoder_to_bf16, L.decoder_silu_mul,
                    L.decoder_qkv_post):
             fn.restype = i
         _LIB = L
@@ -192,6 +193,17 @@ def block(h, attn, wo, post_norm, w_gate, w_up, w_down, eps):
     _launch("decoder_block", h.data_ptr(), attn.data_ptr(), 1 if attn.dtype is BF16 else 0, wo.data_ptr(),
             post_norm.data_ptr(), w_gate.data_ptr(), w_up.data_ptr(), w_down.data_ptr(), s.data_ptr(), out.data_ptr(),
             rows, D, nq, f, eps)
+    return out
+
+
+def causal(q, k, v, scale):
+    """Causal attention of q [T, Hq, d] over k, v [Hkv, T, d], bf16 and
+    contiguous: [T, Hq, d] bf16; None for the shapes it does not take."""
+    T, hq, d = q.shape
+    if T > 1 << 20 or d not in (64, 128, 256) or not _aligned(q, k, v):
+        return None
+    out = torch.empty_like(q)
+    _launch("decoder_causal", q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), T, hq, k.shape[0], d, scale)
     return out
 
 

@@ -389,25 +389,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 1) tc::tmem_dealloc_pair(tmem, P.tmem_cols);
 }
 
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeFn encode_fn() {
-    static EncodeFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            p = nullptr;
-        return reinterpret_cast<EncodeFn>(p);
-    }();
-    return fn;
-}
-
 // [rows][K] bf16, contiguous; box of 64 x box_rows, 128-byte swizzle, zeros outside.
 bool make_map(CUtensorMap* m, const void* base, int rows, int K, int box_rows) {
-    EncodeFn enc = encode_fn();
+    decoder::EncodeFn enc = decoder::encode_fn();
     const cuuint64_t dims[2] = {cuuint64_t(K), cuuint64_t(rows)};
     const cuuint64_t strides[1] = {cuuint64_t(K) * 2};
     const cuuint32_t box[2] = {64, cuuint32_t(box_rows)}, es[2] = {1, 1};
@@ -419,7 +403,7 @@ bool make_map(CUtensorMap* m, const void* base, int rows, int K, int box_rows) {
 // Gate and up [rows][K] bf16 each as one operand: boxes of 4 groups of 16 rows
 // of gate and the same 16 of up.  See joint().
 bool make_map_joint(CUtensorMap* m, const void* gate, const void* up, int rows, int K) {
-    EncodeFn enc = encode_fn();
+    decoder::EncodeFn enc = decoder::encode_fn();
     const cuuint64_t dims[4] = {cuuint64_t(K), 16, 2, cuuint64_t(rows / 16)};
     const cuuint64_t strides[3] = {cuuint64_t(K) * 2, cuuint64_t(static_cast<const char*>(up) - static_cast<const char*>(gate)),
                                    cuuint64_t(K) * 32};
@@ -527,6 +511,23 @@ int launch(const void* x, const void* w0, const void* w1, GemmParams p, cudaStre
 }  // namespace
 
 namespace decoder {
+
+EncodeFn encode_fn() {
+    static EncodeFn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return reinterpret_cast<EncodeFn>(p);
+    }();
+    return fn;
+}
+
+unsigned* error_word() {
+    void* p = nullptr;
+    return cudaGetSymbolAddress(&p, g_error) == cudaSuccess ? static_cast<unsigned*>(p) : nullptr;
+}
 
 bool gemm_takes(int M, int N, int K) {
     // TMA rows are multiples of 16 bytes.

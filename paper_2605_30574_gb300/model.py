@@ -253,12 +253,18 @@ class RandomDecoder:
                 # straight into the stores
                 q = torch.empty((h.shape[0], dims.num_q_heads, dims.head_dim), dtype=torch.bfloat16, device=h.device)
                 self._qkv_into(l, h, pos, q, kl.transpose(0, 1), vl.transpose(0, 1))
-                kh, vh = kl[None], vl[None]
+                kh, vh = kl, vl
             else:
                 q, k, v = self.qkv(l, h, pos)               # [T_p, H, d]
                 kl.copy_(k.transpose(0, 1))
                 vl.copy_(v.transpose(0, 1))
-                kh, vh = k.transpose(0, 1)[None], v.transpose(0, 1)[None]
+                kh, vh = k.transpose(0, 1), v.transpose(0, 1)
+            if q.dtype is kh.dtype is vh.dtype is torch.bfloat16 and K.plain((q,), ()):
+                a = K.causal(q, kh.contiguous(), vh.contiguous(), self.sm_scale)
+                if a is not None:
+                    h = self.block_out(l, h, a)
+                    continue
+            kh, vh = kh[None], vh[None]
             qh = q.transpose(0, 1)[None]                    # [1, Hq, T_p, d]
             a = torch.nn.functional.scaled_dot_product_attention(qh, kh, vh, is_causal=True, scale=self.sm_scale,
                                                                  enable_gqa=G > 1)

@@ -231,3 +231,48 @@ def test_layer_on_fused_projections_and_on_the_librarys(rows, ffn):
     assert torch.equal(h, kept) and got.data_ptr() != h.data_ptr()
     assert (got - want).abs().max() <= 4 * ULP * (want - h).abs().max()
     K.check_device_error()
+
+
+# one row; edges of a key block and of a tile of rows; many tiles; every head
+# dim, with one and more query heads to a kv head
+@pytest.mark.parametrize("T", [1, 63, 64, 65, 127, 128, 129, 200, 1000])
+@pytest.mark.parametrize("hq,hkv,d", [(3, 3, 64), (8, 2, 128), (7, 1, 256)])
+def test_causal_attention(T, hq, hkv, d):
+    """Probabilities and outputs are rounded to bf16, whose eight significant
+    bits put a rounded value within 2^-8 of it each time; a score of d
+    exact products is off by at most 2^-21 of the sum of their magnitudes, and
+    its probability by as much again."""
+    g = gen(T + d)
+    q, k, v = randn(g, T, hq, d), randn(g, hkv, T, d), randn(g, hkv, T, d)
+    k[:, -1] *= 6                     # a later maximum far above the earlier ones
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    got = K.causal(q, k, v, d ** -0.5)
+    K.check_device_error()
+    kd, vd = (x.double().repeat_interleave(hq // hkv, 0) for x in (k, v))
+    qd = q.double().transpose(0, 1)
+    z = (qd @ kd.transpose(1, 2) * d ** -0.5).masked_fill(torch.ones(T, T, device="cuda").triu(1).bool(), float("-inf"))
+    w = torch.softmax(z, -1)
+    want, size = (w @ vd).transpose(0, 1), (w @ vd.abs()).transpose(0, 1)
+    mag = (qd.abs() @ kd.abs().transpose(1, 2) * d ** -0.5).amax(-1).t()[..., None]
+    bound = (2.0 ** -8 + 2 * 2.0 ** -21 * mag + 2.0 ** -19) * size
+    bound = bound + 2.0 ** -8 * (want.abs() + bound) + 1e-30
+    assert bool(((got.double() - want).abs() <= bound).all())
+
+
+def test_causal_attention_rows_do_not_see_later_ones():
+    g = gen(5)
+    q, k, v = (randn(g, *s, dtype=torch.bfloat16) for s in ((300, 4, 128), (2, 300, 128), (2, 300, 128)))
+    want = K.causal(q, k, v, 0.1)
+    k[:, 256:], v[:, 256:] = float("inf"), float("nan")
+    assert torch.equal(K.causal(q, k, v, 0.1)[:256], want[:256])
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(32, 8, 64), (32, 8, 128), (16, 2, 256)])
+def test_causal_attention_is_the_same_every_time(hq, hkv, d):
+    """Every SM full, its CTAs at every distance from one another."""
+    g = gen(d)
+    q, k, v = (randn(g, *s, dtype=torch.bfloat16) for s in ((1500, hq, d), (hkv, 1500, d), (hkv, 1500, d)))
+    want = K.causal(q, k, v, d ** -0.5)
+    for _ in range(20):
+        assert torch.equal(K.causal(q, k, v, d ** -0.5), want)
+    K.check_device_error()
