@@ -2,8 +2,8 @@
 
 * ``libsplice.so``        -- the spliced decode-attention library (C ABI in
   ``include/splice.h``), from ``csrc/``.
-* ``decoder/libsplice_decoder.so`` -- the decoder's projections and
-  elementwise kernels.
+* ``decoder/libsplice_decoder.so`` -- the decoder's projections, prefill
+  attention and elementwise kernels.
 * ``synth/libsplice_synth.so`` -- the device twin of the seeded input generator.
 
 Each translation unit is compiled by its own ``nvcc`` process, in parallel,

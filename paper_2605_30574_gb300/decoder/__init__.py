@@ -1,4 +1,4 @@
-"""ctypes binding of the decoder's elementwise kernels (``libsplice_decoder.so``).
+"""ctypes binding of the decoder's kernels (``libsplice_decoder.so``).
 
 ``model.py`` calls these in place of the torch expressions next to them
 whenever nothing but the values is asked for (``plain``): eager CUDA tensors

@@ -1,7 +1,8 @@
 // Elementwise and normalisation kernels of the decoder that drives Algorithm 1
 // (model.py): RMSNorm, the per-head norm and RoPE of q and k, the residual
 // additions, SwiGLU's product and the attention output's conversion.  The
-// projections between them are library GEMMs, the decode attention is
+// projections between them are gemm.cu's (library GEMMs for shapes that those
+// do not take), the prefill's attention is causal.cu's, the decode attention
 // libsplice.so's.
 //
 // Every kernel reads its inputs once and writes its outputs once, computes in
@@ -13,8 +14,9 @@
 // At a decode batch each of them moves 10-50 MB: one wave or a few of blocks
 // that are bound by their loads' latency, not by bandwidth.  Their point is
 // their number: in a Qwen3-8B-shaped layer of 512 cells they take the place
-// of 62 launches by 7 (980 -> 317 us; a step of two layers and the head 2149
-// -> 797, a prefill of 1024 tokens 2376 -> 890).  Times below are a launch's
+// of 62 launches by 7 (980 -> 317 us with library GEMMs; a step of two layers and
+// the head 2149 -> 797, a prefill of 1024 tokens 2376 -> 890; 216, 700 and 774
+// with gemm.cu and causal.cu).  Times below are a launch's
 // on cold caches at 512 rows of 4096 (32 + 2 x 8 heads of 128, F = 12288).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

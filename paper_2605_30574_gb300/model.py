@@ -20,9 +20,10 @@ Real weights are out of scope: the weights are seeded random normals, so the
 tokens mean nothing; what the run exercises is the propagation of the
 splice through real forward passes (generated-span K/V that depend on the
 spliced attention of every earlier layer and step), which the synthetic
-inputs of the attention benchmark abstract away.  The projections, norms,
-RoPE and MLP are plain torch (cuBLAS GEMMs); every decode attention is the
-library's.
+inputs of the attention benchmark abstract away.  Every decode attention is
+the library's; the prefill's attention, projections, norms, RoPE and MLP are
+the kernels of ``decoder/`` on eager CUDA tensors of the decoder's own types,
+and the plain torch expressions that they stand in for elsewhere.
 """
 from __future__ import annotations
 
