@@ -14,8 +14,8 @@
 // so few rows cost few MMAs.  Each CTA of the pair loads its 128 rows of W and
 // half of x's, 64 of K at a time: an SM takes half the bytes of x from L2, and
 // reads half as many from shared memory per MMA, as one CTA to a tile did
-// (512 rows, gate and up of 12288 x 4096: 82 us so, 61.2 in pairs, 1.68
-// PFLOP/s; 2048 rows 1.99).  The grid is one pair to two SMs, each going
+// (512 rows, gate and up of 12288 x 4096: 82 us so, 60 in pairs, 1.7 PFLOP/s;
+// 2048 rows 1.97-1.99).  The grid is one pair to two SMs, each going
 // through its tiles (those of the same rows of W next to one another in time)
 // with two accumulators, a tile's epilogue under the next one's MMAs.  Too few
 // tiles for that share K over the 2 to 4 pairs of a cluster, whose sums are
@@ -31,8 +31,9 @@
 // launch 2.5.  Against the library's GEMMs with decoder.cu's kernels between,
 // two layers of a prefill (d_model 4096, F 12288, 32 heads of 128 and 8 for
 // keys): 768 rows 855 -> 545 us, 1024 858 -> 682, 1536 970 -> 965, 4096 2870 ->
-// 2767; d_model 5120, F 17408: 1024 1054 -> 1066, 4096 4356 -> 4227.  A decoder
-// layer of 512 cells took 317 so, 248 with one CTA to a tile, 218 now.
+// 2767; d_model 5120, F 17408: 1024 1054 -> 1066, 4096 4356 -> 4227 (all before
+// the smaller tiles of the last wave, see plan).  A decoder layer of 512 cells
+// took 317 so, 248 with one CTA to a tile, 215 now.
 //
 // Every wait is bounded; one that runs out sets the error word, and every role
 // leaves its loop (see decoder_error).
@@ -68,6 +69,7 @@ struct GemmParams {
     int M, N, K;
     int mp;                 // rows of x per tile, the MMA's columns: a multiple of 32, 256 at the most
     int tiles, tiles_m;     // of 256 rows of W (gate and up of 128 features); of mp rows of x
+    int tail, tail_mp, tail_m;  // tiles of W from `tail` on are taken tail_mp rows of x at a time, tail_m times
     int kblocks, split;     // K blocks; pairs of CTAs that share them
     int clusters;           // of `split` pairs, in the grid
     int stages, bufs;       // ring; accumulators in TMEM
@@ -145,10 +147,21 @@ __device__ __forceinline__ void store16(const GemmParams& P, int m, int feature,
     }
 }
 
+// Tile t: its tile of W, first row of x and rows of x.
+struct Tile {
+    int n, m0, mp;
+};
+__device__ __forceinline__ Tile tile_of(const GemmParams& P, int t) {
+    const int whole = P.tail * P.tiles_m;
+    if (t < whole) return {t / P.tiles_m, t % P.tiles_m * P.mp, P.mp};
+    t -= whole;
+    return {P.tail + t / P.tail_m, t % P.tail_m * P.tail_mp, P.tail_mp};
+}
+
 template <int MODE, bool JOINT>
 __global__ void __launch_bounds__(kThreads, 1)
-    gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
-                const __grid_constant__ CUtensorMap tm_w1, const GemmParams P) {
+    gemm_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_xt,
+                const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_w1, const GemmParams P) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[2 * kMaxStages + 5];
     __shared__ uint32_t s_tmem;
@@ -197,7 +210,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tmem = s_tmem;
     const int kb0 = P.kblocks * share / P.split, kb1 = P.kblocks * (share + 1) / P.split;
-    const int first = int(blockIdx.x) / (2 * P.split), ntiles = P.tiles * P.tiles_m;
+    const int first = int(blockIdx.x) / (2 * P.split), ntiles = P.tail * P.tiles_m + (P.tiles - P.tail) * P.tail_m;
     const uint32_t quarter = warp & 3;             // TMEM lanes this warp may read
     const uint32_t acc0 = tmem + ((quarter * 32) << 16);
     const int c_first = (warp - 2) / 4, c_step = kOutWarps / 4;   // this warp's 16-row chunks
@@ -218,14 +231,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         int s = 0, issued = 0;
         uint32_t phase = 1;     // a fresh stage is empty
         for (int t = first; t < ntiles && ok; t += P.clusters) {
-            const int n = t / P.tiles_m, m0 = t % P.tiles_m * P.mp + int(odd) * (P.mp / 2);
+            const Tile tile = tile_of(P, t);
+            const int n = tile.n, m0 = tile.m0 + int(odd) * (tile.mp / 2);
+            const bool in_tail = n >= P.tail;
+            const uint32_t bytes = 2 * (kWBytes + uint32_t(tile.mp) * kBK);
             for (int kb = kb0; kb < kb1; ++kb) {
                 ok = __all_sync(0xffffffffu, tc::mbar_wait(empty(s), phase, &s_abort, &g_error, kErrLoad));
                 if (!ok) break;
                 if (leader) {
                     const uint32_t at = sbase + s * P.stage_bytes, bar = lead + 8u * s;
                     const int k = kb * kBK;
-                    if (!odd) tc::mbar_arrive_expect_tx(full(s), 2 * P.stage_bytes);
+                    if (!odd) tc::mbar_arrive_expect_tx(full(s), bytes);
                     if constexpr (MODE != kSwiglu) {
                         tc::tma_load_2d_pair(at, &tm_w, k, n * FEAT + int(odd) * kFeat, bar);
                     } else if constexpr (JOINT) {
@@ -238,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             tc::tma_load_2d_pair(at + g * 4096 + 2048, &tm_w1, k, row, bar);
                         }
                     }
-                    tc::tma_load_2d_pair(at + kWBytes, &tm_x, k, m0, bar);
+                    tc::tma_load_2d_pair(at + kWBytes, in_tail ? &tm_xt : &tm_x, k, m0, bar);
                 }
                 ++issued;
                 if (++s == P.stages) {
@@ -259,7 +275,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (warp == 1) {
         if (!odd) {
             const bool leader = tc::elect_one();
-            const uint32_t idesc = tc::idesc_bf16_f32(2 * kFeat, 0, false) | (uint32_t(P.mp >> 3) << 17);
             const uint64_t w0 = tc::sw128_desc(sbase, 16, 1024), x0 = tc::sw128_desc(sbase + kWBytes, 16, 1024);
             const uint32_t stage_step = P.stage_bytes >> 4;   // descriptor units of 16 bytes
             int s = 0, buf = 0;
@@ -270,6 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t acc = tmem + buf * P.mp;
+                const uint32_t idesc = tc::idesc_bf16_f32(2 * kFeat, 0, false) | (uint32_t(tile_of(P, t).mp >> 3) << 17);
                 for (int kb = kb0; kb < kb1; ++kb) {
                     ok = __all_sync(0xffffffffu, tc::mbar_wait(full(s), phase, &s_abort, &g_error, kErrMma));
                     if (!ok) break;
@@ -312,7 +328,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         for (int t = first; t < ntiles; t += P.clusters) {
-            const int feature = t / P.tiles_m * FEAT + f0, m0 = t % P.tiles_m * P.mp;
+            const Tile tile = tile_of(P, t);
+            const int feature = tile.n * FEAT + f0, m0 = tile.m0, mp = tile.mp;
             if (P.split == 1) {
 #pragma unroll
                 for (int i = 0; i < AHEAD; ++i) load_h<MODE>(P, m0 + 16 * (c_first + i * c_step), feature, h[i]);
@@ -321,15 +338,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) break;
             tc::tc_fence_after();
             if (P.split > 1) break;    // the cluster's one tile: below
-            for (int j = c_first; 16 * j < P.mp; j += AHEAD * c_step) {
+            for (int j = c_first; 16 * j < mp; j += AHEAD * c_step) {
 #pragma unroll
                 for (int i = 0; i < AHEAD; ++i) {
                     const int c = 16 * (j + i * c_step);
-                    if (c >= P.mp) break;
+                    if (c >= mp) break;
                     float v[16];
                     tmem_ld16(acc0 + buf * P.mp + c, v);
                     store16<MODE>(P, m0 + c, feature, v, h[i]);
-                    load_h<MODE>(P, c + 16 * AHEAD * c_step < P.mp ? m0 + c + 16 * AHEAD * c_step : P.M, feature, h[i]);
+                    load_h<MODE>(P, c + 16 * AHEAD * c_step < mp ? m0 + c + 16 * AHEAD * c_step : P.M, feature, h[i]);
                 }
             }
             tc::tc_fence_before();
@@ -418,6 +435,9 @@ struct Resident {
     int n[4];
 };
 
+// A K block of 64 for mp rows of x, in clocks.
+double block_clocks(int mp) { return std::max(2.0 * mp, (16384.0 + 64.0 * mp) / 75.0) + 20.0; }
+
 // The launch's shape (host arithmetic only): tiles of 32 to 256 rows of x and
 // shares of K, of the least time in clocks by what a K block of 64 takes (2 per
 // row of x in MMAs, or its bytes at the 75 a clock that an SM gets from L2),
@@ -428,6 +448,9 @@ void plan(int mode, GemmParams& p, const int (&resident)[4]) {
     const int feat = mode == kSwiglu ? kFeat : 2 * kFeat;
     p.tiles = (p.N + feat - 1) / feat;
     p.kblocks = (p.K + kBK - 1) / kBK;
+    p.tail = p.tiles;
+    p.tail_mp = 32;
+    p.tail_m = 1;
     double least = 0;
     GemmParams best = p;
     for (int mp = 256; mp >= 32; mp -= 32) {
@@ -444,13 +467,34 @@ void plan(int mode, GemmParams& p, const int (&resident)[4]) {
             c.bufs = tiles > c.clusters ? 2 : 1;
             c.tmem_cols = 32;
             while (c.tmem_cols < uint32_t(c.mp * c.bufs)) c.tmem_cols *= 2;
-            const double block = std::max(2.0 * c.mp, (16384.0 + 64.0 * c.mp) / 75.0) + 20.0;
-            const double clocks = double((tiles + c.clusters - 1) / c.clusters) * block * c.kblocks / c.split + 8.0 * c.mp / c.split +
-                                  (c.split > 1 ? 6000.0 : 0.0);
+            const double clocks = double((tiles + c.clusters - 1) / c.clusters) * block_clocks(c.mp) * c.kblocks / c.split +
+                                  8.0 * c.mp / c.split + (c.split > 1 ? 6000.0 : 0.0);
             if (least == 0 || clocks < least) {
                 least = clocks;
                 best = c;
             }
+        }
+        // The tiles past the last whole wave, in smaller ones that make up
+        // one wave (4096 deep, gate and up of 12288: 512 rows, 2.53 waves, 63.7
+        // -> 61.8 us; 1024, 5.05 waves, 117.9 -> 111.9; 6144 features, 2048
+        // rows 60.9 -> 56.1; 4096 by 12288 deep, 2048 rows 136 -> 122).
+        c.split = 1;
+        c.clusters = resident[0];
+        const long waves = tiles / c.clusters;
+        if (waves < 1 || tiles % c.clusters == 0) continue;
+        c.tail = int(waves * c.clusters / c.tiles_m);
+        c.bufs = 2;
+        c.tmem_cols = 32;
+        while (c.tmem_cols < uint32_t(c.mp * c.bufs)) c.tmem_cols *= 2;
+        for (c.tail_mp = 32; c.tail_mp < mp; c.tail_mp += 32) {
+            c.tail_m = (p.M + c.tail_mp - 1) / c.tail_mp;
+            if (long(c.tail) * c.tiles_m + long(c.tiles - c.tail) * c.tail_m > (waves + 1) * c.clusters) continue;
+            const double clocks = (waves * block_clocks(mp) + block_clocks(c.tail_mp)) * c.kblocks + 8.0 * mp;
+            if (clocks < least) {
+                least = clocks;
+                best = c;
+            }
+            break;
         }
     }
     p = best;
@@ -486,8 +530,10 @@ int launch(const void* x, const void* w0, const void* w1, GemmParams p, cudaStre
         return r;
     }();
     plan(MODE, p, resident.n);
-    CUtensorMap mx, m0, m1;
+    CUtensorMap mx, mt, m0, m1;
     if (!make_map(&mx, x, p.M, p.K, p.mp / 2)) return int(cudaErrorInvalidValue);
+    mt = mx;
+    if (p.tail < p.tiles && !make_map(&mt, x, p.M, p.K, p.tail_mp / 2)) return int(cudaErrorInvalidValue);
     if (!(JOINT ? make_map_joint(&m0, w0, w1, p.N, p.K) : make_map(&m0, w0, p.N, p.K, MODE == kSwiglu ? 16 : kFeat)))
         return int(cudaErrorInvalidValue);
     m1 = m0;
@@ -505,7 +551,7 @@ int launch(const void* x, const void* w0, const void* w1, GemmParams p, cudaStre
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return int(cudaLaunchKernelEx(&cfg, gemm_kernel<MODE, JOINT>, mx, m0, m1, p));
+    return int(cudaLaunchKernelEx(&cfg, gemm_kernel<MODE, JOINT>, mx, mt, m0, m1, p));
 }
 
 }  // namespace
@@ -565,7 +611,8 @@ int decoder_gemm(int mode, const void* x, const void* w0, const void* w1, const 
 // CTAs are resident together, for tests (no CUDA call): out = {rows of x per
 // tile, K blocks, shares of K, tiles of W, tiles of rows of x, clusters, ring
 // stages, bytes per stage, TMEM columns, accumulators, bytes of the sums traded,
-// shared memory}.
+// shared memory, tiles of W before the tail, the tail's rows of x per tile, and
+// tiles of rows of x}.
 int decoder_gemm_plan(int mode, int M, int N, int K, const int* resident, long* out) {
     if (mode < 0 || mode > 2 || resident[0] < 1 || !decoder::gemm_takes(M, N, K)) return int(cudaErrorInvalidValue);
     GemmParams p{};
@@ -575,9 +622,9 @@ int decoder_gemm_plan(int mode, int M, int N, int K, const int* resident, long* 
     const int r[4] = {resident[0], resident[1], resident[2], resident[3]};
     plan(mode, p, r);
     const long traded = p.split > 1 ? long(p.split) * ((p.mp / 16 + p.split - 1) / p.split) * kChunkBytes : 0;
-    const long v[12] = {p.mp, p.kblocks, p.split, p.tiles, p.tiles_m, p.clusters, p.stages, long(p.stage_bytes),
-                        long(p.tmem_cols), p.bufs, traded, long(p.stages) * long(p.stage_bytes) + 1024};
-    for (int i = 0; i < 12; ++i) out[i] = v[i];
+    const long v[15] = {p.mp, p.kblocks, p.split, p.tiles, p.tiles_m, p.clusters, p.stages, long(p.stage_bytes),
+                        long(p.tmem_cols), p.bufs, traded, long(p.stages) * long(p.stage_bytes) + 1024, p.tail, p.tail_mp, p.tail_m};
+    for (int i = 0; i < 15; ++i) out[i] = v[i];
     return 0;
 }
 

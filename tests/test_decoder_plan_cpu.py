@@ -15,7 +15,7 @@ def lib():
 
 
 def test_every_launch_fits(lib):
-    out = (ctypes.c_long * 12)()
+    out = (ctypes.c_long * 15)()
     for mode in (0, 1, 2):
         for room in ((76, 36, 23, 15), (74, 36, 22, 14), (10, 4, 0, 0), (1, 0, 0, 0)):
             resident = (ctypes.c_int * 4)(*room)
@@ -23,7 +23,7 @@ def test_every_launch_fits(lib):
                 for N in (1, 8, 127, 128, 129, 640, 2000, 4096, 6144, 12288, 40000, 151936):
                     for k in (8, 64, 72, 504, 512, 1000, 1024, 4096, 12288, 20000):
                         assert lib.decoder_gemm_plan(mode, M, N, k, resident, out) == 0
-                        mp, kblocks, split, tiles, tiles_m, clusters, stages, stage, cols, bufs, traded, smem = out
+                        mp, kblocks, split, tiles, tiles_m, clusters, stages, stage, cols, bufs, traded, smem, tail, tail_mp, tail_m = out
                         feat = 128 if mode == 2 else 256
                         assert mp % 32 == 0 and 32 <= mp <= 256 and tiles_m * mp >= M > (tiles_m - 1) * mp
                         assert tiles * feat >= N > (tiles - 1) * feat and kblocks * 64 >= k > (kblocks - 1) * 64
@@ -33,6 +33,12 @@ def test_every_launch_fits(lib):
                         # an accumulator to spare where a pair has a second tile
                         assert cols <= 512 and cols & (cols - 1) == 0 and mp * bufs <= cols
                         assert bufs == (2 if tiles * tiles_m > clusters else 1)
+                        # the tail: smaller tiles, of all rows, that fill one wave at the most
+                        assert 0 <= tail <= tiles and tail_mp % 32 == 0 and 32 <= tail_mp <= mp
+                        if tail < tiles:
+                            waves = tiles * tiles_m // clusters
+                            assert split == 1 and tail_m * tail_mp >= M > (tail_m - 1) * tail_mp and bufs == 2
+                            assert waves * clusters < tail * tiles_m + (tiles - tail) * tail_m <= (waves + 1) * clusters
                         # a stage holds W's and half of x's block; the ring the sums that the pairs trade
                         assert stage == 16384 + mp * 64 and stage % 1024 == 0 and stages >= 2
                         chunks = mp // 16
