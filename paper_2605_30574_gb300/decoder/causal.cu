@@ -162,6 +162,12 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
             tc::mbar_wait(kfull(i & 1), uint32_t(i >> 1) & 1u, &no_abort, err, kErrDrain);
             tc::mbar_wait(vfull(i & 1), uint32_t(i >> 1) & 1u, &no_abort, err, kErrDrain);
         }
+        // So must the commits arrive: the last P V's comes after the stages',
+        // but nothing says that two commits arrive in their order.
+        bool ok = j == nblk;
+        for (int i = max(0, j - 2); ok && i < j; ++i)
+            ok = tc::mbar_wait(kempty(i & 1), uint32_t(i >> 1) & 1u, &s_abort, err, kErrDrain) &&
+                 tc::mbar_wait(vempty(i & 1), uint32_t(i >> 1) & 1u, &s_abort, err, kErrDrain);
     } else if (warp == kMmaWarp) {
         const bool leader = tc::elect_one();
         constexpr uint32_t idesc_qk = tc::idesc_bf16_f32(kRows, kBN, false), idesc_pv = tc::idesc_bf16_f32(kRows, D, true);

@@ -272,6 +272,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tc::mbar_wait(full(j % P.stages), uint32_t(j / P.stages) & 1u, &no_abort, &g_error, kErrDrain);
             }
         }
+        // So must the even CTA's commits arrive on this CTA's barriers: the
+        // sums' commit comes after the stages', but nothing says that two
+        // commits arrive in their order.
+        for (int j = max(0, issued - P.stages); ok && j < issued; ++j)
+            ok = tc::mbar_wait(empty(j % P.stages), uint32_t(j / P.stages) & 1u, &s_abort, &g_error, kErrDrain);
     } else if (warp == 1) {
         if (!odd) {
             const bool leader = tc::elect_one();

@@ -210,6 +210,26 @@ def test_fused_projection_rows_are_independent():
     assert not bool(got[7].isfinite().any()) and bool(got[12].isnan().all())
 
 
+def test_fused_projections_behind_one_another():
+    """Launches of every kind of shape in a row, so that one's CTAs come to SMs
+    that another's have just left: each gives the bits it gives alone."""
+    g = gen(9)
+    cases = []
+    for M, N, k in ((1, 4096, 4096), (16, 640, 1000), (64, 6144, 512), (257, 4096, 512), (400, 20000, 136), (3, 130, 72)):
+        x, w = randn(g, M, k, dtype=torch.bfloat16), randn(g, N, k, dtype=torch.bfloat16)
+        cases.append((x, w, gemm(1, x, w).float()))
+    outs = []
+    for i in range(60):
+        x, w, want = cases[i * 5 % len(cases)]
+        y = torch.empty_like(want)
+        assert K.lib().decoder_gemm(1, x.data_ptr(), w.data_ptr(), None, None, y.data_ptr(), *want.shape, x.shape[1],
+                                    torch.cuda.current_stream().cuda_stream) == 0
+        outs.append((y, want))
+    K.check_device_error()
+    for y, want in outs:
+        assert torch.equal(y, want)
+
+
 # one row; a tile of rows, two; shares of K; more tiles than pairs of CTAs;
 # many rows; rows of the MLP that TMA does not take
 @pytest.mark.parametrize("rows,ffn", [(1, 1544), (128, 1544), (257, 1544), (300, 12288), (1030, 1544), (9000, 12288),
