@@ -180,7 +180,7 @@ class RandomDecoder:
             return False
         if pos is None:
             return (w["wo"].shape == (D, nq) and w["post_norm"].shape == (D,)
-                    and w["w_gate"].shape == w["w_up"].shape == w["w_down"].shape[::-1]
+                    and w["w_gate"].shape == w["w_up"].shape == w["w_down"].shape[::-1] and w["w_gate"].shape[1:] == (D,)
                     and K.plain((h,), (w["wo"], w["post_norm"], w["w_gate"], w["w_up"], w["w_down"])))
         return (d in (64, 128, 256) and h.dim() >= 2 and pos.dtype in K.POSITIONS and pos.shape == h.shape[:-1]
                 and self.inv_freq.dtype is torch.float32 and self.inv_freq.shape == (d // 2,)

@@ -12,6 +12,7 @@ import math
 import pytest
 import torch
 
+from paper_2605_30574_gb300 import decoder as K
 from paper_2605_30574_gb300.model import RandomDecoder, donor_tokens, tiny_dims
 from paper_2605_30574_gb300.synth import workloads as W
 
@@ -74,3 +75,18 @@ def test_prefill_is_causal(model):
     assert torch.equal(k1[:, :, :-1], k2[:, :, :-1]) and torch.equal(v1[:, :, :-1], v2[:, :, :-1])
     assert not torch.equal(k1[:, :, -1], k2[:, :, -1])
     assert not torch.equal(l1, l2)
+
+
+# An MLP of another input width has no kernels: the torch expressions refuse it.
+@pytest.mark.parametrize("gate,up,down", [((512, 128), (512, 128), (128, 512)), ((512, 320), (512, 320), (320, 512)),
+                                          ((512, 256), (512, 128), (256, 512)), ((512, 256), (512, 256), (128, 512))])
+def test_kernels_take_only_an_mlp_of_the_models_width(model, monkeypatch, gate, up, down):
+    monkeypatch.setattr(K, "plain", lambda acts, weights: True)
+    h = torch.zeros(3, model.dims.d_model)
+    assert model._kernels(0, h)
+    kept = dict(model.layers[0])
+    for n, shape in (("w_gate", gate), ("w_up", up), ("w_down", down)):
+        monkeypatch.setitem(model.layers[0], n, torch.zeros(shape, dtype=torch.bfloat16))
+    assert not model._kernels(0, h)
+    monkeypatch.undo()
+    assert all(model.layers[0][n] is kept[n] for n in kept)
