@@ -22,6 +22,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "decoder.h"
 
 namespace {
@@ -217,8 +219,8 @@ struct alignas(2 * V) Vec {
 // elements V i .. V i + V - 1 of both halves of the head (V = D / 64), so the
 // rotation needs no exchange.  4 bytes per element and one head per warp, so
 // that a row's 48 heads are in flight at once: 8.0 us, where torch made 36
-// launches.  Pointers are 16-byte aligned and strides
-// multiples of 8 (the caller checks).
+// launches.  Rows of heads and the norms' weights are
+// read and written V elements at a time: see qkv_post_takes.
 template <int D>
 __global__ void __launch_bounds__(kThreads)
     qkv_post_kernel(HeadRows q, HeadRows k, HeadRows v, const __nv_bfloat16* __restrict__ q_norm,
@@ -316,6 +318,16 @@ size_t align256(size_t n) { return (n + 255) / 256 * 256; }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Whether every word of d / 64 elements that qkv_post_kernel<d> takes is aligned.
+bool qkv_post_takes(std::initializer_list<const void*> ptrs, const long* strides, int n_strides, int d) {
+    if (d != 64 && d != 128 && d != 256) return false;
+    for (const void* p : ptrs)
+        if (reinterpret_cast<uintptr_t>(p) % unsigned(d / 32)) return false;
+    for (int i = 0; i < n_strides; ++i)
+        if (strides[i] % (d / 64)) return false;
+    return true;
+}
+
 }  // namespace
 
 // Every call returns the cudaError_t of its launches and takes contiguous rows
@@ -369,8 +381,8 @@ int decoder_qkv_post(const void* q, const void* k, const void* v, void* q_out, v
     const HeadRows a{static_cast<const bf*>(q), strides[0], static_cast<bf*>(q_out), strides[3], strides[4]};
     const HeadRows b{static_cast<const bf*>(k), strides[1], static_cast<bf*>(k_out), strides[5], strides[6]};
     const HeadRows c{static_cast<const bf*>(v), strides[2], static_cast<bf*>(v_out), strides[7], strides[8]};
+    if (!qkv_post_takes({q, k, v, q_out, k_out, v_out, q_norm, k_norm}, strides, 9, d)) return int(cudaErrorInvalidValue);
     auto kernel = d == 64 ? qkv_post_kernel<64> : (d == 128 ? qkv_post_kernel<128> : qkv_post_kernel<256>);
-    if (d != 64 && d != 128 && d != 256) return int(cudaErrorInvalidValue);
     const dim3 grid(unsigned(rows), unsigned((Hq + 2 * Hkv + kThreads / 32 - 1) / (kThreads / 32)));
     return launch(kernel, grid, static_cast<cudaStream_t>(stream), a, b, c, static_cast<const bf*>(q_norm),
                   static_cast<const bf*>(k_norm), static_cast<const float*>(inv_freq), pos, pos_kind, Hq, Hkv, eps);
@@ -396,7 +408,8 @@ int decoder_qkv(const void* h, const void* in_norm, const void* wqkv, void* scra
                 const long* strides, const void* q_norm, const void* k_norm, const void* inv_freq, const void* pos,
                 int pos_kind, long rows, int D, int Hq, int Hkv, int d, float eps, void* stream) {
     const int nq = Hq * d, nk = Hkv * d, n = nq + 2 * nk;
-    if (!aligned16(wqkv) || !aligned16(scratch)) return int(cudaErrorInvalidValue);
+    if (!aligned16(wqkv) || !aligned16(scratch) || !qkv_post_takes({q_out, k_out, v_out, q_norm, k_norm}, strides, 6, d))
+        return int(cudaErrorInvalidValue);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     bf* x = static_cast<bf*>(scratch);
     bf* y = reinterpret_cast<bf*>(static_cast<char*>(scratch) + align256(size_t(rows) * D * 2));

@@ -187,7 +187,8 @@ class RandomDecoder:
                 and w["in_norm"].shape == (D,) and w["q_norm"].shape == w["k_norm"].shape == (d,)
                 and w["wq"].shape == (nq, D) and w["wk"].shape == w["wv"].shape == (nk, D)
                 and K.plain((h, pos, self.inv_freq),
-                            (w["in_norm"], w["wq"], w["wk"], w["wv"], w["q_norm"], w["k_norm"])))
+                            (w["in_norm"], w["wq"], w["wk"], w["wv"], w["q_norm"], w["k_norm"]))
+                and w["q_norm"].data_ptr() % (d // 32) == w["k_norm"].data_ptr() % (d // 32) == 0)
 
     def _attn_ok(self, h: torch.Tensor, attn: torch.Tensor) -> bool:
         """Whether the attention output is laid out as the kernels read it."""

@@ -51,3 +51,28 @@ def test_every_launch_fits(lib):
     room = (ctypes.c_int * 4)(76, 36, 23, 15)
     for bad in ((0, 0, 8, 8), (0, 65537, 8, 8), (0, 1, 0, 8), (0, 1, 8, 12), (3, 1, 8, 8), (-1, 1, 8, 8)):
         assert lib.decoder_gemm_plan(*bad, room, out) != 0
+
+
+def test_misaligned_words_are_refused_before_any_launch(lib):
+    """Every pointer and stride that is read or written in words of d / 64
+    elements, one at a time off by an element."""
+    for d in (128, 256):
+        ok = [1 << 20] * 6                       # (never read: each call is refused)
+        norms = [1 << 20] * 2
+
+        def post(ptrs, strides, norms):
+            return lib.decoder_qkv_post(*ptrs, (ctypes.c_long * 9)(*strides), *norms, 1 << 20, 1 << 20, 0, 1, 1, 1, d, 1e-6, 0)
+
+        def off(values, i, by):
+            return [v + by * (j == i) for j, v in enumerate(values)]
+
+        for i in range(6):
+            assert post(off(ok, i, 2), [d] * 9, norms) == 1
+        for i in range(9):
+            assert post(ok, off([d] * 9, i, 1), norms) == 1
+        for i in range(2):
+            assert post(ok, [d] * 9, off(norms, i, 2)) == 1
+            one = off(norms, i, 2)
+            assert lib.decoder_qkv(1 << 20, 1 << 20, 1 << 20, 1 << 20, *ok[:3], (ctypes.c_long * 6)(*[d] * 6), *one,
+                                   1 << 20, 1 << 20, 0, 1, 64, 1, 1, d, 1e-6, 0) == 1
+    assert lib.decoder_qkv_post(*[1 << 20] * 6, (ctypes.c_long * 9)(*[96] * 9), *[1 << 20] * 4, 0, 1, 1, 1, 96, 1e-6, 0) == 1

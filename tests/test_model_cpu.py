@@ -13,7 +13,7 @@ import pytest
 import torch
 
 from paper_2605_30574_gb300 import decoder as K
-from paper_2605_30574_gb300.model import RandomDecoder, donor_tokens, tiny_dims
+from paper_2605_30574_gb300.model import DecoderDims, RandomDecoder, donor_tokens, tiny_dims
 from paper_2605_30574_gb300.synth import workloads as W
 
 
@@ -90,3 +90,17 @@ def test_kernels_take_only_an_mlp_of_the_models_width(model, monkeypatch, gate, 
     assert not model._kernels(0, h)
     monkeypatch.undo()
     assert all(model.layers[0][n] is kept[n] for n in kept)
+
+
+# The kernel reads the head norms' weights in words of d / 64 elements: views
+# that do not start on one (of a flat buffer of all parameters, say) are torch's.
+@pytest.mark.parametrize("d", [64, 128, 256])
+@pytest.mark.parametrize("name", ["q_norm", "k_norm"])
+def test_kernels_take_only_head_norms_on_whole_words(monkeypatch, d, name):
+    monkeypatch.setattr(K, "plain", lambda acts, weights: True)
+    model = RandomDecoder(DecoderDims(1, 2, 1, d, 64, 64, 8), device="cpu")
+    h, pos = torch.zeros(3, 64), torch.arange(3)
+    flat = torch.ones(d + 8, dtype=torch.bfloat16)
+    for at in range(8):
+        model.layers[0][name] = flat[at:at + d]
+        assert model._kernels(0, h, pos) == (at % (d // 64) == 0)
