@@ -23,6 +23,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "../csrc/tc_ptx.cuh"
 #include "decoder.h"
@@ -362,10 +363,12 @@ int launch(const void* q, const void* k, const void* v, void* out, int T, int Hq
 
 extern "C" {
 
-// See the head of this file; 16-byte aligned.  Returns a cudaError_t.
+// See the head of this file; 16-byte aligned; a positive, finite scale.  Returns a
+// cudaError_t.
 int decoder_causal(const void* q, const void* k, const void* v, void* out, long T, int Hq, int Hkv, int d, float scale,
                    void* stream) {
-    if (T < 1 || T > (1 << 20) || Hq < 1 || Hkv < 1 || Hq % Hkv != 0) return int(cudaErrorInvalidValue);
+    if (T < 1 || T > (1 << 20) || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || !(scale > 0.f && scale < INFINITY))
+        return int(cudaErrorInvalidValue);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (d == 64) return launch<64>(q, k, v, out, int(T), Hq, Hkv, scale, st);
     if (d == 128) return launch<128>(q, k, v, out, int(T), Hq, Hkv, scale, st);

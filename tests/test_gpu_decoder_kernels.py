@@ -161,6 +161,30 @@ def test_prefill_into_stores_and_into_copies(hq, hkv, d, T):
     assert torch.equal(k.float(), kf) and torch.equal(v.float(), vf) and torch.equal(got, want)
 
 
+def on_cpu(model):
+    """The same decoder on the CPU, where every piece is a torch expression."""
+    m = RandomDecoder(model.dims, device="cpu")
+    m.embed, m.final_norm, m.lm_head, m.inv_freq = (t.cpu() for t in (model.embed, model.final_norm, model.lm_head,
+                                                                       model.inv_freq))
+    m.layers = [{n: w.cpu() for n, w in layer.items()} for layer in model.layers]
+    m.sm_scale = model.sm_scale
+    return m
+
+
+@pytest.mark.parametrize("scale", [0.0, -0.0, -0.1, 0.1])
+def test_prefill_at_any_scale(scale):
+    """sm_scale is the caller's to set.  Both ways round bf16 a dozen times a
+    layer (2^-9 each, on values of the logits' own spread)."""
+    model = RandomDecoder(DecoderDims(2, 4, 2, 64, 256, 320, 60), seed=3, std=0.06)
+    model.sm_scale = scale
+    tokens = torch.randint(0, 60, (150,), generator=gen(1), device="cuda")
+    k, v = (torch.zeros(2, 2, 150, 64, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    got = model.prefill(tokens, k, v).cpu()
+    want = on_cpu(model).prefill(tokens.cpu(), k.cpu(), v.cpu())
+    assert bool(got.isfinite().all())
+    assert (got - want).norm() <= 24 * 2.0 ** -9 * want.norm()
+
+
 def gemm(mode, x, w0, w1=None, h=None):
     M, k, N = x.shape[0], x.shape[1], w0.shape[0]
     y = torch.full((M + 1, N), float("nan"), dtype=torch.float32 if mode == 1 else torch.bfloat16, device="cuda")
