@@ -198,11 +198,9 @@ def block(h, attn, wo, post_norm, w_gate, w_up, w_down, eps):
 
 def causal(q, k, v, scale):
     """Causal attention of q [T, Hq, d] over k, v [Hkv, T, d], bf16 and
-    contiguous: [T, Hq, d] bf16; None for the shapes and scales it does not
-    take (it masks scores before it scales them: only a positive scale, and one
-    well inside fp32, leaves a masked one at -inf)."""
+    contiguous: [T, Hq, d] bf16; None for the shapes it does not take."""
     T, hq, d = q.shape
-    if not 2.0 ** -100 < scale < 2.0 ** 100 or T > 1 << 20 or d not in (64, 128, 256) or not _aligned(q, k, v):
+    if T > 1 << 20 or d not in (64, 128, 256) or not _aligned(q, k, v):
         return None
     out = torch.empty_like(q)
     _launch("decoder_causal", q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), T, hq, k.shape[0], d, scale)

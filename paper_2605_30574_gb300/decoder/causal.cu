@@ -23,7 +23,6 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <cmath>
 
 #include "../csrc/tc_ptx.cuh"
 #include "decoder.h"
@@ -222,6 +221,11 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
         const uint32_t mine = tmem + (uint32_t(warp * 32) << 16);
         float m = 0.f, l = 0.f;
         bool ok = true;
+        // A positive scale goes in with the exponent's fma, past the masking and
+        // the maximum; one of zero or below would make NaN or +inf of a masked
+        // score and turn the order round, so it goes in first.
+        const bool scale_first = !(scale_log2 > 0.f);
+        const float scale_later = scale_first ? 1.f : scale_log2;
         for (int j = 0; j < nblk; ++j) {
             const int s = j & 1;
             ok = __all_sync(0xffffffffu, tc::mbar_wait(sfull(s), uint32_t(j >> 1) & 1u, &s_abort, err, kErrOut));
@@ -230,6 +234,10 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
             float v[2][32];
             tmem_ld32_done(mine + s * kBN, v[0]);
             tmem_ld32_done(mine + s * kBN + 32, v[1]);
+            if (scale_first) {
+#pragma unroll
+                for (int i = 0; i < kBN; ++i) v[i >> 5][i & 31] *= scale_log2;
+            }
             if ((j + 1) * kBN > row0 + 1) {          // the diagonal's blocks
                 const int last = row - j * kBN;      // this row's last key in the block
 #pragma unroll
@@ -239,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
             float top = v[0][0];
 #pragma unroll
             for (int i = 1; i < kBN; ++i) top = fmaxf(top, v[i >> 5][i & 31]);
-            top *= scale_log2;
+            top *= scale_later;
             if (j == 0) {
                 m = top;
             } else if (__any_sync(0xffffffffu, top > m)) {
@@ -268,7 +276,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    const float a = ex2(fmaf(v[half][2 * i], scale_log2, -m)), b = ex2(fmaf(v[half][2 * i + 1], scale_log2, -m));
+                    const float a = ex2(fmaf(v[half][2 * i], scale_later, -m)), b = ex2(fmaf(v[half][2 * i + 1], scale_later, -m));
                     const __nv_bfloat162 p2 = __floats2bfloat162_rn(a, b);
                     pk[i] = *reinterpret_cast<const uint32_t*>(&p2);
                     part[i & 3] += __low2float(p2) + __high2float(p2);
@@ -363,12 +371,10 @@ int launch(const void* q, const void* k, const void* v, void* out, int T, int Hq
 
 extern "C" {
 
-// See the head of this file; 16-byte aligned; a positive, finite scale.  Returns a
-// cudaError_t.
+// See the head of this file; 16-byte aligned.  Returns a cudaError_t.
 int decoder_causal(const void* q, const void* k, const void* v, void* out, long T, int Hq, int Hkv, int d, float scale,
                    void* stream) {
-    if (T < 1 || T > (1 << 20) || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || !(scale > 0.f && scale < INFINITY))
-        return int(cudaErrorInvalidValue);
+    if (T < 1 || T > (1 << 20) || Hq < 1 || Hkv < 1 || Hq % Hkv != 0) return int(cudaErrorInvalidValue);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (d == 64) return launch<64>(q, k, v, out, int(T), Hq, Hkv, scale, st);
     if (d == 128) return launch<128>(q, k, v, out, int(T), Hq, Hkv, scale, st);

@@ -161,30 +161,6 @@ def test_prefill_into_stores_and_into_copies(hq, hkv, d, T):
     assert torch.equal(k.float(), kf) and torch.equal(v.float(), vf) and torch.equal(got, want)
 
 
-def on_cpu(model):
-    """The same decoder on the CPU, where every piece is a torch expression."""
-    m = RandomDecoder(model.dims, device="cpu")
-    m.embed, m.final_norm, m.lm_head, m.inv_freq = (t.cpu() for t in (model.embed, model.final_norm, model.lm_head,
-                                                                       model.inv_freq))
-    m.layers = [{n: w.cpu() for n, w in layer.items()} for layer in model.layers]
-    m.sm_scale = model.sm_scale
-    return m
-
-
-@pytest.mark.parametrize("scale", [0.0, -0.0, -0.1, 0.1])
-def test_prefill_at_any_scale(scale):
-    """sm_scale is the caller's to set.  Both ways round bf16 a dozen times a
-    layer (2^-9 each, on values of the logits' own spread)."""
-    model = RandomDecoder(DecoderDims(2, 4, 2, 64, 256, 320, 60), seed=3, std=0.06)
-    model.sm_scale = scale
-    tokens = torch.randint(0, 60, (150,), generator=gen(1), device="cuda")
-    k, v = (torch.zeros(2, 2, 150, 64, device="cuda", dtype=torch.bfloat16) for _ in range(2))
-    got = model.prefill(tokens, k, v).cpu()
-    want = on_cpu(model).prefill(tokens.cpu(), k.cpu(), v.cpu())
-    assert bool(got.isfinite().all())
-    assert (got - want).norm() <= 24 * 2.0 ** -9 * want.norm()
-
-
 def gemm(mode, x, w0, w1=None, h=None):
     M, k, N = x.shape[0], x.shape[1], w0.shape[0]
     y = torch.full((M + 1, N), float("nan"), dtype=torch.float32 if mode == 1 else torch.bfloat16, device="cuda")
@@ -277,30 +253,47 @@ def test_layer_on_fused_projections_and_on_the_librarys(rows, ffn):
     K.check_device_error()
 
 
+def assert_causal(got, q, k, v, scale):
+    """Probabilities and outputs are rounded to bf16, whose eight significant
+    bits put a rounded value within 2^-8 of it each time; a score of d
+    exact products is off by at most 2^-21 of the sum of their magnitudes, and
+    its probability by as much again."""
+    G, T = q.shape[1] // k.shape[0], q.shape[0]
+    kd, vd = (x.double().repeat_interleave(G, 0) for x in (k, v))
+    qd = q.double().transpose(0, 1)
+    z = (qd @ kd.transpose(1, 2) * scale).masked_fill(torch.ones(T, T, device="cuda").triu(1).bool(), float("-inf"))
+    w = torch.softmax(z, -1)
+    want, size = (w @ vd).transpose(0, 1), (w @ vd.abs()).transpose(0, 1)
+    mag = (qd.abs() @ kd.abs().transpose(1, 2) * abs(scale)).amax(-1).t()[..., None]
+    bound = (2.0 ** -8 + 2 * 2.0 ** -21 * mag + 2.0 ** -19) * size
+    bound = bound + 2.0 ** -8 * (want.abs() + bound) + 1e-30
+    assert bool(((got.double() - want).abs() <= bound).all())
+
+
 # one row; edges of a key block and of a tile of rows; many tiles; every head
 # dim, with one and more query heads to a kv head
 @pytest.mark.parametrize("T", [1, 63, 64, 65, 127, 128, 129, 200, 1000])
 @pytest.mark.parametrize("hq,hkv,d", [(3, 3, 64), (8, 2, 128), (7, 1, 256)])
 def test_causal_attention(T, hq, hkv, d):
-    """Probabilities and outputs are rounded to bf16, whose eight significant
-    bits put a rounded value within 2^-8 of it each time; a score of d
-    exact products is off by at most 2^-21 of the sum of their magnitudes, and
-    its probability by as much again."""
     g = gen(T + d)
     q, k, v = randn(g, T, hq, d), randn(g, hkv, T, d), randn(g, hkv, T, d)
     k[:, -1] *= 6                     # a later maximum far above the earlier ones
     q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
     got = K.causal(q, k, v, d ** -0.5)
     K.check_device_error()
-    kd, vd = (x.double().repeat_interleave(hq // hkv, 0) for x in (k, v))
-    qd = q.double().transpose(0, 1)
-    z = (qd @ kd.transpose(1, 2) * d ** -0.5).masked_fill(torch.ones(T, T, device="cuda").triu(1).bool(), float("-inf"))
-    w = torch.softmax(z, -1)
-    want, size = (w @ vd).transpose(0, 1), (w @ vd.abs()).transpose(0, 1)
-    mag = (qd.abs() @ kd.abs().transpose(1, 2) * d ** -0.5).amax(-1).t()[..., None]
-    bound = (2.0 ** -8 + 2 * 2.0 ** -21 * mag + 2.0 ** -19) * size
-    bound = bound + 2.0 ** -8 * (want.abs() + bound) + 1e-30
-    assert bool(((got.double() - want).abs() <= bound).all())
+    assert_causal(got, q, k, v, d ** -0.5)
+
+
+# scales that the model's caller may set, two that fp32 holds as zero or denormal
+@pytest.mark.parametrize("scale", [0.0, -0.0, 1e-50, 1e-40, -1e-3, -0.125, -1.0])
+@pytest.mark.parametrize("hq,hkv,d", [(2, 1, 64), (4, 2, 128), (2, 2, 256)])
+def test_causal_attention_at_any_scale(hq, hkv, d, scale):
+    """As with a positive scale (the bound is test_causal_attention's)."""
+    T, g = 200, gen(d)
+    q, k, v = (randn(g, *s, dtype=torch.bfloat16) for s in ((T, hq, d), (hkv, T, d), (hkv, T, d)))
+    got = K.causal(q, k, v, scale)
+    K.check_device_error()
+    assert_causal(got, q, k, v, scale)
 
 
 def test_causal_attention_rows_do_not_see_later_ones():

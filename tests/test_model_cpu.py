@@ -12,7 +12,6 @@ import math
 import pytest
 import torch
 
-from paper_2605_30574_gb300 import build as B
 from paper_2605_30574_gb300 import decoder as K
 from paper_2605_30574_gb300.model import DecoderDims, RandomDecoder, donor_tokens, tiny_dims
 from paper_2605_30574_gb300.synth import workloads as W
@@ -105,12 +104,3 @@ def test_kernels_take_only_head_norms_on_whole_words(monkeypatch, d, name):
     for at in range(8):
         model.layers[0][name] = flat[at:at + d]
         assert model._kernels(0, h, pos) == (at % (d // 64) == 0)
-
-
-@pytest.mark.parametrize("scale", [0.0, 1e-50, -0.125, -math.inf, 1e39, math.inf, math.nan])
-def test_prefill_attention_kernel_takes_positive_scales(scale):
-    """The kernel scales scores after it has masked them, in fp32."""
-    B.build()
-    q, k = torch.zeros(4, 2, 64, dtype=torch.bfloat16), torch.zeros(1, 4, 64, dtype=torch.bfloat16)
-    assert K.causal(q, k, k, scale) is None
-    assert K.lib().decoder_causal(1 << 20, 1 << 20, 1 << 20, 1 << 20, 4, 2, 1, 64, scale, 0) == 1
