@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
             if (j == 0) {
                 m = top;
             } else if (__any_sync(0xffffffffu, top > m)) {
-                const float to = fmaxf(m, top), alpha = ex2(m - to);
+                const float to = fmaxf(m, top), alpha = ex2(m - (to == -INFINITY ? 0.f : to));
                 m = to;
                 l *= alpha;
                 // O is at rest: the last P V issued is the previous block's
@@ -268,6 +268,8 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
                 }
                 tc::tmem_wait_st();
             }
+            // a row whose every score so far is -inf has no weights yet
+            const float ref = m == -INFINITY ? 0.f : m;
             // (the weights as they are used, rounded: their sum then makes up
             // for part of the rounding)
             float part[4] = {0.f, 0.f, 0.f, 0.f};
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
                 uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    const float a = ex2(fmaf(v[half][2 * i], scale_later, -m)), b = ex2(fmaf(v[half][2 * i + 1], scale_later, -m));
+                    const float a = ex2(fmaf(v[half][2 * i], scale_later, -ref)), b = ex2(fmaf(v[half][2 * i + 1], scale_later, -ref));
                     const __nv_bfloat162 p2 = __floats2bfloat162_rn(a, b);
                     pk[i] = *reinterpret_cast<const uint32_t*>(&p2);
                     part[i & 3] += __low2float(p2) + __high2float(p2);
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<D>::CTAS)
         if (ok) ok = __all_sync(0xffffffffu, tc::mbar_wait(pvdone, uint32_t(nblk - 1) & 1u, &s_abort, err, kErrOut));
         if (ok) {
             tc::tc_fence_after();
-            const float inv = 1.f / l;
+            const float inv = l == 0.f ? 0.f : 1.f / l;   // (no weights at all: zeros)
             uint4* dst = reinterpret_cast<uint4*>(out + (size_t(row) * Hq + head) * D);
 #pragma unroll
             for (int c = 0; c < D; c += 32) {

@@ -304,6 +304,22 @@ def test_causal_attention_rows_do_not_see_later_ones():
     assert torch.equal(K.causal(q, k, v, 0.1)[:256], want[:256])
 
 
+# some keys of the first block, all of it, more, and more than a tile of rows
+@pytest.mark.parametrize("ruled_out", [10, 64, 70, 200])
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_causal_attention_over_keys_that_are_ruled_out(ruled_out, d):
+    """A key whose score is -inf weighs nothing, also where a row has met no
+    other yet; a row that meets no other at all gives zeros."""
+    g = gen(d)
+    q, k, v = (randn(g, *s, dtype=torch.bfloat16) for s in ((260, 2, d), (1, 260, d), (1, 260, d)))
+    q[:, :, 0] = 1
+    k[:, :ruled_out, 0] = float("-inf")
+    got = K.causal(q, k, v, d ** -0.5)
+    K.check_device_error()
+    assert not bool(got[:ruled_out].any())
+    assert_causal(got[ruled_out:], q[ruled_out:], k[:, ruled_out:], v[:, ruled_out:], d ** -0.5)
+
+
 @pytest.mark.parametrize("hq,hkv,d", [(32, 8, 64), (32, 8, 128), (16, 2, 256)])
 def test_causal_attention_is_the_same_every_time(hq, hkv, d):
     """Every SM full, its CTAs at every distance from one another."""
