@@ -86,11 +86,13 @@ def build(force: bool = False, verbose: bool = False) -> None:
     headers = sorted(glob.glob(os.path.join(csrc, "*.h")) + glob.glob(os.path.join(csrc, "*.cuh")) +
                      glob.glob(os.path.join(ROOT, "include", "*.h")))
     synth_src = [os.path.join(PKG, "synth", "synth.cu")]
+    decoder_headers = [os.path.join(csrc, "tc_ptx.cuh"), os.path.join(csrc, "per_device.h"),
+                       os.path.join(PKG, "decoder", "decoder.h")]
     decoder_src = sorted(glob.glob(os.path.join(PKG, "decoder", "*.cu")))
     with cf.ThreadPoolExecutor(max_workers=3) as ex:
         a = ex.submit(build_lib, "splice", sources, headers, splice_lib_path(), force, verbose)
         b = ex.submit(build_lib, "synth", synth_src, [], synth_lib_path(), force, verbose)
-        c = ex.submit(build_lib, "decoder", decoder_src, [os.path.join(csrc, "tc_ptx.cuh"), os.path.join(PKG, "decoder", "decoder.h")], decoder_lib_path(), force, verbose)
+        c = ex.submit(build_lib, "decoder", decoder_src, decoder_headers, decoder_lib_path(), force, verbose)
         a.result()
         b.result()
         c.result()

@@ -24,6 +24,7 @@
 
 #include <algorithm>
 
+#include "../csrc/per_device.h"
 #include "../csrc/tc_ptx.cuh"
 #include "decoder.h"
 
@@ -347,12 +348,16 @@ bool make_map(CUtensorMap* m, const void* base, int x, int y, int z, size_t sy, 
 template <int D>
 int launch(const void* q, const void* k, const void* v, void* out, int T, int Hq, int Hkv, float scale, cudaStream_t st) {
     using C = Cfg<D>;
-    static const bool attr = [] {
-        return cudaFuncSetAttribute(causal_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM)) == cudaSuccess;
-    }();
+    static splice::PerDevice<bool> kept;
+    bool set = false;
+    const cudaError_t e = kept.get(&set, [](int, bool* done) {
+        *done = true;
+        return cudaFuncSetAttribute(causal_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(C::SMEM));
+    });
+    if (e != cudaSuccess) return int(e);
     unsigned* err = decoder::error_word();
     CUtensorMap mq, mk, mv;
-    if (!attr || !err || !make_map(&mq, q, D, Hq, T, D, size_t(Hq) * D, 1, kRows) ||
+    if (!err || !make_map(&mq, q, D, Hq, T, D, size_t(Hq) * D, 1, kRows) ||
         !make_map(&mk, k, D, T, Hkv, D, size_t(T) * D, kBN, 1) || !make_map(&mv, v, D, T, Hkv, D, size_t(T) * D, kBN, 1))
         return int(cudaErrorInvalidValue);
     cudaLaunchConfig_t cfg = {};

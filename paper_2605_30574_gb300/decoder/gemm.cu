@@ -45,6 +45,7 @@
 
 #include <algorithm>
 
+#include "../csrc/per_device.h"
 #include "../csrc/tc_ptx.cuh"
 #include "decoder.h"
 
@@ -515,10 +516,11 @@ bool joint(const void* gate, const void* up, int rows) {
 
 template <int MODE, bool JOINT>
 int launch(const void* x, const void* w0, const void* w1, GemmParams p, cudaStream_t st) {
-    static const Resident resident = [] {
-        Resident r{};
-        cudaFuncSetAttribute(gemm_kernel<MODE, JOINT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-        for (int i = 0; i < 4; ++i) {
+    static splice::PerDevice<Resident> kept;
+    Resident resident;
+    const cudaError_t e = kept.get(&resident, [](int, Resident* r) {
+        cudaError_t err = cudaFuncSetAttribute(gemm_kernel<MODE, JOINT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+        for (int i = 0; i < 4 && err == cudaSuccess; ++i) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(2u * (i + 1));
             cfg.blockDim = dim3(kThreads);
@@ -529,11 +531,12 @@ int launch(const void* x, const void* w0, const void* w1, GemmParams p, cudaStre
             attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
             cfg.attrs = &attr;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&r.n[i], gemm_kernel<MODE, JOINT>, &cfg) != cudaSuccess) r.n[i] = 0;
+            err = cudaOccupancyMaxActiveClusters(&r->n[i], gemm_kernel<MODE, JOINT>, &cfg);
         }
-        r.n[0] = std::max(r.n[0], 1);
-        return r;
-    }();
+        r->n[0] = std::max(r->n[0], 1);
+        return err;
+    });
+    if (e != cudaSuccess) return int(e);
     plan(MODE, p, resident.n);
     CUtensorMap mx, mt, m0, m1;
     if (!make_map(&mx, x, p.M, p.K, p.mp / 2)) return int(cudaErrorInvalidValue);

@@ -329,3 +329,16 @@ def test_causal_attention_is_the_same_every_time(hq, hkv, d):
     for _ in range(20):
         assert torch.equal(K.causal(q, k, v, d ** -0.5), want)
     K.check_device_error()
+
+
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="one device")
+def test_a_second_device():
+    """Both devices of a process, one after the other."""
+    outs = []
+    for dev in range(2):
+        with torch.cuda.device(dev):
+            model = RandomDecoder(DecoderDims(1, 4, 2, 128, 256, 512, 60), device=f"cuda:{dev}")
+            k, v = (torch.zeros(1, 2, 70, 128, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+            outs.append(model.prefill(torch.arange(70, device="cuda") % 60, k, v).cpu())
+            K.check_device_error()
+    assert torch.equal(*outs)
