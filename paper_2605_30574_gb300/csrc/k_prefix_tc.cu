@@ -48,6 +48,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "per_device.h"
 #include "splice_internal.h"
 #include "tc_ptx.cuh"
 
@@ -994,13 +995,13 @@ EncodeFn encode_fn() {
 template <int D, bool SHORT>
 int launch_d(const TcParams& tp, const CUtensorMap* m, cudaStream_t st, bool overlap_previous) {
     using C = Cfg<D, SHORT>;
-    static int sms = 0;
-    if (!sms) {
-        cudaFuncSetAttribute(prefix_tc_kernel<D, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
+    static PerDevice<int> kept;
+    int sms = 0;
+    const cudaError_t e = kept.get(&sms, [](int dev, int* n) {
+        const cudaError_t err = cudaFuncSetAttribute(prefix_tc_kernel<D, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        return err != cudaSuccess ? err : cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+    });
+    if (e != cudaSuccess) return int(e);
     const int most = tp.a.prefix_ctas > 0 && tp.a.prefix_ctas < sms ? tp.a.prefix_ctas : sms;
     const unsigned grid = unsigned(tp.n_items < most ? tp.n_items : most);
     if (!overlap_previous) {

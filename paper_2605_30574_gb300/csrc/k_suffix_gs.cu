@@ -37,6 +37,7 @@
 #include <cmath>
 
 #include "gs_common.cuh"
+#include "per_device.h"
 #include "tc_ptx.cuh"
 
 namespace splice {
@@ -709,17 +710,22 @@ __global__ void __launch_bounds__(GS<D, GT>::WARPS * 32)
 template <int D, int GT>
 int launch_gs_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap_previous) {
     using C = GS<D, GT>;
-    static int blocks_per_sm = 0, sms = 0;
-    if (!blocks_per_sm) {
-        cudaFuncSetAttribute(gs_kernel<D, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, gs_kernel<D, GT>, C::WARPS * 32, C::SMEM);
-        if (blocks_per_sm < 1) blocks_per_sm = 1;
-    }
+    struct Device {
+        int sms, blocks_per_sm;
+    };
+    static PerDevice<Device> kept;
+    Device on{};
+    const cudaError_t e = kept.get(&on, [](int dev, Device* s) {
+        cudaError_t err = cudaFuncSetAttribute(gs_kernel<D, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        if (err == cudaSuccess) err = cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev);
+        if (err == cudaSuccess)
+            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s->blocks_per_sm, gs_kernel<D, GT>, C::WARPS * 32, C::SMEM);
+        if (s->blocks_per_sm < 1) s->blocks_per_sm = 1;
+        return err;
+    });
+    if (e != cudaSuccess) return int(e);
     const long want = (long(n_items) + C::WARPS - 1) / C::WARPS;
-    const long cap = long(blocks_per_sm) * sms;
+    const long cap = long(on.blocks_per_sm) * on.sms;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(want < cap ? want : cap));
     cfg.blockDim = dim3(C::WARPS * 32);
@@ -730,7 +736,7 @@ int launch_gs_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap_
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = overlap_previous ? 1 : 0;
-    return int(cudaLaunchKernelEx(&cfg, gs_kernel<D, GT>, p, n_items, sms));
+    return int(cudaLaunchKernelEx(&cfg, gs_kernel<D, GT>, p, n_items, on.sms));
 }
 
 }  // namespace

@@ -46,6 +46,7 @@
 #include <cmath>
 
 #include "gs_common.cuh"
+#include "per_device.h"
 #include "tc_ptx.cuh"
 
 namespace splice {
@@ -822,13 +823,13 @@ struct Shape {
 template <int D, int NT>
 int launch_mma_t(const AttnParams& p, int n_items, cudaStream_t st, bool overlap_previous) {
     using C = GM<D, NT>;
-    static int sms = 0;
-    if (!sms) {
-        cudaFuncSetAttribute(gs_mma_kernel<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
+    static PerDevice<int> kept;
+    int sms = 0;
+    const cudaError_t e = kept.get(&sms, [](int dev, int* n) {
+        const cudaError_t err = cudaFuncSetAttribute(gs_mma_kernel<D, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        return err != cudaSuccess ? err : cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+    });
+    if (e != cudaSuccess) return int(e);
     Shape<D, NT> sh(p.gs_rows);
     // few items: spread over the SMs rather than a CTA's warps
     sh.warps = int(std::min<long>(sh.warps, (long(n_items) + sms - 1) / sms));

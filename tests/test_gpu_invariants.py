@@ -263,3 +263,18 @@ def test_attention_reads_the_entry_appended_right_before():
     ref = oracle_rows(wl, inp, sb.seqs, l, t, range(sb.B))
     assert_close(out, ref, f"older slot l={l} t={t}")
     S.splice_check_device_error(sb.desc)
+
+
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="one device")
+def test_a_second_device():
+    """Both devices of a process, one after the other: every generated-span
+    kernel (one row, several, rows of 256 dims) and the prompt-span pass."""
+    for hq, hkv, d in ((4, 4, 64), (8, 2, 128), (4, 2, 256)):
+        wl = WL.Workload("two", 1, hq, hkv, d, 2, 300, (WL.SAME_ALGO, WL.ZERO), 12, (0, 1), (0, 5), 8, 4, batch=10 ** 6)
+        outs = []
+        for dev in range(2):
+            with torch.cuda.device(dev):
+                a = SweepBatch(wl, seqs=wl.sequences())
+                outs.append(a.run(0, 7).cpu())
+                S.splice_check_device_error(a.desc)
+        assert torch.equal(*outs)
