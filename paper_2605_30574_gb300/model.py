@@ -182,7 +182,7 @@ class RandomDecoder:
             return (w["wo"].shape == (D, nq) and w["post_norm"].shape == (D,)
                     and w["w_gate"].shape == w["w_up"].shape == w["w_down"].shape[::-1] and w["w_gate"].shape[1:] == (D,)
                     and K.plain((h,), (w["wo"], w["post_norm"], w["w_gate"], w["w_up"], w["w_down"])))
-        return (d in (64, 128, 256) and h.dim() >= 2 and pos.dtype in K.POSITIONS and pos.shape == h.shape[:-1]
+        return (d in (64, 128, 256) and _own(self, "rope") and h.dim() >= 2 and pos.dtype in K.POSITIONS and pos.shape == h.shape[:-1]
                 and self.inv_freq.dtype is torch.float32 and self.inv_freq.shape == (d // 2,)
                 and w["in_norm"].shape == (D,) and w["q_norm"].shape == w["k_norm"].shape == (d,)
                 and w["wq"].shape == (nq, D) and w["wk"].shape == w["wv"].shape == (nk, D)
@@ -251,7 +251,7 @@ class RandomDecoder:
         h = self.embed[tokens].float()
         for l in range(dims.num_layers):
             kl, vl = k_out[l], v_out[l]                     # [Hkv, T_p, d]
-            if type(self).qkv is RandomDecoder.qkv and self._kernels(l, h, pos) and self._store_ok(h, kl, vl):
+            if _own(self, "qkv") and self._kernels(l, h, pos) and self._store_ok(h, kl, vl):
                 # straight into the stores
                 q = torch.empty((h.shape[0], dims.num_q_heads, dims.head_dim), dtype=torch.bfloat16, device=h.device)
                 self._qkv_into(l, h, pos, q, kl.transpose(0, 1), vl.transpose(0, 1))
@@ -272,6 +272,15 @@ class RandomDecoder:
                                                                  enable_gqa=G > 1)
             h = self.block_out(l, h, a[0].transpose(0, 1).contiguous())
         return self.logits(h[-1])
+
+
+_PIECES = {name: getattr(RandomDecoder, name) for name in ("rope", "qkv")}
+
+
+def _own(model: RandomDecoder, name: str) -> bool:
+    """Whether a piece of the decoder is the one above, which the kernels stand
+    in for, and not a subclass's or an instance's own."""
+    return getattr(getattr(model, name), "__func__", None) is _PIECES[name]
 
 
 def donor_tokens(prompt: torch.Tensor, kind: int, gen: torch.Generator, vocab: int, scaffold_head: int,

@@ -13,7 +13,7 @@ import pytest
 import torch
 
 from paper_2605_30574_gb300 import decoder as K
-from paper_2605_30574_gb300.model import DecoderDims, RandomDecoder, donor_tokens, tiny_dims
+from paper_2605_30574_gb300.model import DecoderDims, RandomDecoder, _own, donor_tokens, tiny_dims
 from paper_2605_30574_gb300.synth import workloads as W
 
 
@@ -104,3 +104,40 @@ def test_kernels_take_only_head_norms_on_whole_words(monkeypatch, d, name):
     for at in range(8):
         model.layers[0][name] = flat[at:at + d]
         assert model._kernels(0, h, pos) == (at % (d // 64) == 0)
+
+
+def test_a_piece_of_ones_own_is_the_one_that_runs(monkeypatch):
+    """A decoder that brings its own rope or qkv -- by a subclass, on an
+    instance, or patched into the class -- is not passed by."""
+    calls = []
+
+    class Unturned(RandomDecoder):
+        def rope(self, x, pos):
+            calls.append("rope")
+            return x
+
+    class Spy(RandomDecoder):
+        def qkv(self, l, h, pos):
+            calls.append("qkv")
+            return super().qkv(l, h, pos)
+
+    dims = DecoderDims(1, 2, 1, 64, 64, 64, 8)
+    tokens, h, pos = torch.arange(5), torch.zeros(5, 64), torch.arange(5)
+    stores = [torch.zeros(1, 1, 5, 64, dtype=torch.bfloat16) for _ in range(2)]
+    plain, a, b, c = (cls(dims, device="cpu") for cls in (RandomDecoder, Unturned, RandomDecoder, Spy))
+    b.rope = lambda x, pos: calls.append("rope") or x
+    for m in (a, b):
+        m.qkv(0, h, pos)
+        m.prefill(tokens, *stores)
+    c.prefill(tokens, *stores)
+    assert calls == ["rope"] * 8 + ["qkv"]
+    monkeypatch.setattr(K, "plain", lambda acts, weights: True)
+    assert plain._kernels(0, h, pos) and c._kernels(0, h, pos)
+    assert not a._kernels(0, h, pos) and not b._kernels(0, h, pos)
+    assert _own(plain, "qkv") and _own(a, "qkv") and not _own(c, "qkv")
+    b.qkv = b.qkv
+    assert _own(b, "qkv")
+    b.qkv = lambda l, h, pos: None
+    assert not _own(b, "qkv")
+    monkeypatch.setattr(RandomDecoder, "rope", Unturned.rope)
+    assert not plain._kernels(0, h, pos)
