@@ -63,14 +63,19 @@ def plain(acts, weights) -> bool:
         return False
     grad = torch.is_grad_enabled()
     for t in acts:
-        if type(t) is not torch.Tensor or t.device != dev or not t.is_contiguous() or (grad and t.requires_grad) \
-                or t.numel() == 0:
+        if type(t) is not torch.Tensor or not _values(t, dev) or (grad and t.requires_grad):
             return False
     for t in weights:
-        if t.dtype is not BF16 or t.device != dev or not t.is_contiguous() or (grad and t.requires_grad) \
-                or type(t) not in (torch.Tensor, torch.nn.Parameter):
+        if t.dtype is not BF16 or type(t) not in (torch.Tensor, torch.nn.Parameter) or not _values(t, dev) \
+                or (grad and t.requires_grad):
             return False
     return True
+
+
+def _values(t, dev) -> bool:
+    """Whether the tensor's values are what lies at its address: not those of a
+    negated view, nor none (an empty tensor, one of zeros without memory)."""
+    return t.device == dev and t.is_contiguous() and not t.is_neg() and t.numel() > 0 and t.data_ptr() != 0
 
 
 def joined(*ws):

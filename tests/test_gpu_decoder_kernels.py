@@ -149,6 +149,26 @@ def test_transforms_modes_and_other_types_take_the_torch_path():
     assert tangent.abs().max() > 0
 
 
+def test_tensors_whose_values_are_not_at_their_address_take_the_torch_path():
+    model = RandomDecoder(DecoderDims(1, 4, 2, 64, 128, 64, 50), seed=0)
+    h, pos = randn(gen(), 6, 128), torch.arange(6, device="cuda")
+    negated, nothing = torch._neg_view(h), torch._efficientzerotensor((6, 128), device="cuda")
+    for x in (negated, nothing):
+        assert not model._kernels(0, x, pos) and not model._kernels(0, x) and not K.plain((x,), ())
+    for got, want in zip(model.qkv(0, negated, pos), model.qkv(0, -h, pos)):
+        close(got, want, scale=2 * want.abs().amax(-1, keepdim=True).expand_as(want))
+    weight = torch._neg_view(model.layers[0]["wo"])
+    assert not K.plain((h,), (weight,))
+
+
+def test_an_mlp_of_no_width():
+    """The torch expressions add nothing for it; a kernel has nothing to launch."""
+    model = RandomDecoder(DecoderDims(1, 2, 1, 64, 128, 0, 50), seed=0)
+    h, attn = randn(gen(), 6, 128), randn(gen(1), 6, 2, 64)
+    want = model.block_out(0, h.clone().requires_grad_(), attn).detach()
+    close(model.block_out(0, h, attn), want, scale=want.abs().amax().expand_as(want))
+
+
 @pytest.mark.parametrize("hq,hkv,d,T", [(1, 1, 64, 1), (6, 2, 128, 77), (4, 4, 256, 130)])
 def test_prefill_into_stores_and_into_copies(hq, hkv, d, T):
     """Straight into contiguous bf16 stores, and through copies into others."""
