@@ -199,6 +199,8 @@ class RandomDecoder:
     def _store_ok(self, h: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> bool:
         """Whether the kernels may write k and v of the rows h to these stores."""
         shape = (self.dims.num_kv_heads, h.shape[0], self.dims.head_dim)
+        if (k.is_inference() or v.is_inference()) and not torch.is_inference_mode_enabled():
+            return False                                    # (torch's copy refuses those)
         return (k.dtype is v.dtype is torch.bfloat16 and k.shape == v.shape == shape and K.plain((k, v), ())
                 and k.device == h.device and k.data_ptr() % 16 == v.data_ptr() % 16 == 0)
 
@@ -255,6 +257,8 @@ class RandomDecoder:
                 # straight into the stores
                 q = torch.empty((h.shape[0], dims.num_q_heads, dims.head_dim), dtype=torch.bfloat16, device=h.device)
                 self._qkv_into(l, h, pos, q, kl.transpose(0, 1), vl.transpose(0, 1))
+                for t in (kl, vl):
+                    torch.autograd.graph.increment_version(t)   # (as a copy into them would)
                 kh, vh = kl, vl
             else:
                 q, k, v = self.qkv(l, h, pos)               # [T_p, H, d]

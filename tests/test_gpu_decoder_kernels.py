@@ -181,6 +181,27 @@ def test_prefill_into_stores_and_into_copies(hq, hkv, d, T):
     assert torch.equal(k.float(), kf) and torch.equal(v.float(), vf) and torch.equal(got, want)
 
 
+def test_prefill_writes_its_stores_as_torch_does():
+    """A graph that saved a store sees that it was written since; a store of
+    inference mode is refused outside it."""
+    model = RandomDecoder(DecoderDims(1, 2, 1, 64, 128, 64, 50), seed=0)
+    tokens = torch.arange(9, device="cuda")
+    k, v = (torch.zeros(1, 1, 9, 64, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    for store in (k, v):
+        x = torch.ones(64, device="cuda", dtype=torch.bfloat16, requires_grad=True)
+        y = (x * store).sum()
+        model.prefill(tokens, k, v)
+        with pytest.raises(RuntimeError, match="modified by an inplace operation"):
+            y.backward()
+    with torch.inference_mode():
+        ki, vi = torch.zeros_like(k), torch.zeros_like(v)
+        model.prefill(tokens, ki, vi)
+        assert torch.equal(ki, k) and torch.equal(vi, v)
+    for stores in ((ki, v), (k, vi)):
+        with pytest.raises(RuntimeError, match="inference tensor"):
+            model.prefill(tokens, *stores)
+
+
 def gemm(mode, x, w0, w1=None, h=None):
     M, k, N = x.shape[0], x.shape[1], w0.shape[0]
     y = torch.full((M + 1, N), float("nan"), dtype=torch.float32 if mode == 1 else torch.bfloat16, device="cuda")
