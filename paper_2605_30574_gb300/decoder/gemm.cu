@@ -637,10 +637,11 @@ int decoder_gemm_plan(int mode, int M, int N, int K, const int* resident, long* 
 }
 
 // The error word of the current device's launches (a wait ran out), and
-// clears it; synchronises.
+// clears it; synchronises the device.
 int decoder_error(unsigned* word) {
     const unsigned zero = 0;
-    cudaError_t e = cudaMemcpyFromSymbol(word, g_error, sizeof zero);
+    cudaError_t e = cudaDeviceSynchronize();    // (the copy waits for blocking streams only)
+    if (e == cudaSuccess) e = cudaMemcpyFromSymbol(word, g_error, sizeof zero);
     if (e == cudaSuccess && *word) e = cudaMemcpyToSymbol(g_error, &zero, sizeof zero);
     return int(e);
 }

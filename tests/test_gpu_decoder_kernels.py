@@ -383,3 +383,16 @@ def test_a_second_device():
             outs.append(model.prefill(torch.arange(70, device="cuda") % 60, k, v).cpu())
             K.check_device_error()
     assert torch.equal(*outs)
+
+
+def test_the_error_check_waits_for_every_stream():
+    """Launches on a side stream, whose streams torch makes non-blocking, may
+    still set the word."""
+    K.check_device_error()
+    side, done = torch.cuda.Stream(), torch.cuda.Event()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(200_000_000)          # some 0.1 s
+        done.record()
+    assert not done.query()
+    K.check_device_error()
+    assert done.query()
