@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 import torch
 import torch.autograd.forward_ad as _fwad
@@ -229,10 +230,48 @@ def logits(x, w):
     return y
 
 
+# The error word of a device is one for all its launches, and reading it clears
+# it: what has been read is kept here, device by device, so that every reader
+# sees it.
+_records: dict = {}
+_records_lock = threading.Lock()
+
+
+class ErrorReader:
+    """Whether a bounded wait of a launch on the current device ran out since the
+    reader last asked (or was made, with ``fresh``; else ever): each reader is
+    told once, whoever reads the word first, and also of others' launches,
+    which the word does not tell apart."""
+
+    def __init__(self, fresh: bool = True):
+        self._seen = {}
+        if fresh:
+            self._take()
+
+    def _take(self):
+        """Synchronises the device, moves its word to the record and returns
+        what this reader has not seen of it."""
+        device, word = torch.cuda.current_device(), ctypes.c_uint()
+        with _records_lock:
+            record = _records.setdefault(device, [])
+            rc = lib().decoder_error(ctypes.byref(word))
+            if rc != 0:
+                raise RuntimeError(f"decoder kernels: CUDA error {rc}")
+            if word.value:
+                record.append(word.value)
+            at, self._seen[device] = self._seen.get(device, 0), len(record)
+            return record[at:]
+
+    def check(self):
+        """Raises if one did; synchronises the device."""
+        words = self._take()
+        if words:
+            raise RuntimeError("decoder kernels: error word " + ", ".join(f"0x{w:x}" for w in words))
+
+
+_reader = ErrorReader(fresh=False)
+
+
 def check_device_error():
-    """Raises if a bounded wait of an earlier launch on the current device ran
-    out (and clears the record); synchronises."""
-    word = ctypes.c_uint()
-    rc = lib().decoder_error(ctypes.byref(word))
-    if rc != 0 or word.value:
-        raise RuntimeError(f"decoder kernels: CUDA error {rc}, error word 0x{word.value:x}")
+    """The check of one reader that all callers of this function share."""
+    _reader.check()

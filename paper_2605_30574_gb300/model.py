@@ -246,7 +246,9 @@ class RandomDecoder:
     def prefill(self, tokens: torch.Tensor, k_out: torch.Tensor, v_out: torch.Tensor) -> torch.Tensor:
         """Causal forward of one token sequence [T_p] at positions 0..T_p-1.
         Writes every layer's RoPE'd K and V into k_out, v_out [N][Hkv][T_p][d]
-        and returns the last position's logits [vocab]."""
+        and returns the last position's logits [vocab].  Does not wait for the
+        GPU: a bounded wait that ran out (the outputs are then wrong) shows in
+        ``decoder.check_device_error``, also for the pieces above."""
         dims = self.dims
         G = dims.num_q_heads // dims.num_kv_heads
         pos = torch.arange(tokens.shape[0], device=self.device)
@@ -340,6 +342,8 @@ class SpliceDecode:
         gen.manual_seed(seed + 1)
         self.y0 = torch.empty(P, dtype=torch.long, device=dev)
         self.donor_prompts = {}
+        with torch.cuda.device(dev):
+            self._errors = K.ErrorReader()
         for p in range(P):
             self.y0[p] = model.prefill(prompts[p], self.k_clean[p], self.v_clean[p]).argmax()
             for i, k in enumerate(self.stored):
@@ -356,11 +360,21 @@ class SpliceDecode:
         self.ws = torch.empty(S.splice_workspace_bytes(self.desc), dtype=torch.uint8, device=dev)
         self.out = torch.empty((self.B, dims.num_q_heads, d), dtype=torch.float32, device=dev)
         self.first_token = self.y0[torch.tensor([q.prompt for q in self.seqs], device=dev)]
+        self.check()
+
+    def check(self):
+        """Raises if a bounded wait of a kernel ran out (its outputs are then
+        wrong) since the last check; synchronises the device.  Called at the
+        end of the prefills and of ``decode``; for ``step``, by its caller."""
+        S.splice_check_device_error(self.desc)
+        with torch.cuda.device(self.model.device):
+            self._errors.check()
 
     @torch.no_grad()
     def step(self, t: int, tokens: torch.Tensor) -> torch.Tensor:
         """Forward pass of step t (1 <= t < T): tokens [B] are y_{t-1}; returns
-        the logits [B][vocab] whose argmax is y_t."""
+        the logits [B][vocab] whose argmax is y_t.  Does not wait for the GPU:
+        see ``check``."""
         model, dims = self.model, self.model.dims
         pos = torch.full((self.B,), self.Tp + t - 1, device=model.device)
         h = model.embed[tokens].float()
@@ -386,8 +400,7 @@ class SpliceDecode:
                 done |= toks[-1] == eos
                 y = torch.where(done, torch.full_like(y, eos), y)
             toks.append(y)
-        S.splice_check_device_error(self.desc)
-        K.check_device_error()
+        self.check()
         return torch.stack(toks, dim=1)
 
     def close(self):
@@ -450,7 +463,7 @@ def main(argv=None):
     torch.cuda.synchronize()
     prof = S.splice_profile_read(run.desc)
     S.splice_profile_enable(run.desc, False)
-    S.splice_check_device_error(run.desc)
+    run.check()
     attn_ms = sum(v[1] for v in prof.values())
     print(json.dumps({
         "what": "Algorithm 1 greedy decode, random-init Qwen3-8B-shaped decoder, ladder batch 0",

@@ -16,6 +16,7 @@ import torch
 
 import oracle
 from paper_2605_30574_gb300 import build as B
+from paper_2605_30574_gb300 import decoder as K
 from paper_2605_30574_gb300.model import RandomDecoder, SpliceDecode, tiny_dims
 from paper_2605_30574_gb300.synth import workloads as WL
 
@@ -121,3 +122,27 @@ def test_splice_changes_patched_cells_only():
     l0 = run.step(1, toks[:, 0])
     assert not torch.equal(l0[2], l0[0]) and not torch.equal(l0[3], l0[0])
     run.close()
+
+
+def test_a_wait_that_ran_out_in_the_prefills_is_reported(monkeypatch):
+    """A prefill's outputs are then wrong; the prefills' end says so (the
+    library's own call, but for the word that it reads)."""
+    real, reads = K.lib(), []
+
+    class Library:
+        def __getattr__(self, name):
+            return getattr(real, name)
+
+        def decoder_error(self, ref):
+            rc = real.decoder_error(ref)
+            reads.append(1)
+            if len(reads) > 1:                  # (the first is the reader's making)
+                ref._obj.value = 0x10
+            return rc
+
+    monkeypatch.setattr(K, "_LIB", Library())
+    monkeypatch.setattr(K, "_records", {})
+    model = RandomDecoder(tiny_dims(), seed=0)
+    prompts = torch.randint(0, model.dims.vocab, (1, 20), device="cuda")
+    with pytest.raises(RuntimeError, match="0x10"):
+        SpliceDecode(model, prompts, (WL.SAME_ALGO, WL.ZERO), [WL.Seq(0, 0, 0, 0)], 4, 2, 2, filler=3)
