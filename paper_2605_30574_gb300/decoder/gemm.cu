@@ -79,9 +79,11 @@ struct GemmParams {
     void* y;
 };
 
-// (a few units of 2^-24 off, far inside the output's bf16 rounding; the exact
-// division and expf cost a tile of 144 rows 3.4 us of its epilogue warps)
-__device__ __forceinline__ float silu(float g) { return __fdividef(g, 1.f + __expf(-g)); }
+// g / (1 + e^-g), a quarter of both so that the divisor stays where the short
+// division works: within 3 units in the last place of the exact division of
+// the same.  That costs 72.2 us against 67.7 for 512 rows of 12288 x 4096, 16.9
+// against 11.6 for 400 of 3072 x 1024; __expf, 67.2, is off by 2 + 1.2 |g| units.
+__device__ __forceinline__ float silu(float g) { return __fdividef(0.25f * g, fmaf(0.25f, expf(-g), 0.25f)); }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];

@@ -237,6 +237,22 @@ def test_fused_projections(M, N, k):
         assert bool(((gemm(2, x, gate, up) - s).abs() <= bound).all())
 
 
+def test_fused_silu_over_its_range():
+    """Gates far below zero too, where e^-g nears and passes fp32's largest value
+    (silu is 0 from there on, as torch's of fp32 is): the output's rounding to
+    bf16, whose eight significant bits put it within 2^-8, and no more.  Gates of bf16 by weights of one and ups of one are exact."""
+    g = torch.linspace(-95, 95, 64 * 64, device="cuda").bfloat16().view(64, 64)
+    g[0, :12] = torch.tensor([-20, -80, -86.5, -87, -87.5, -88, -88.5, -89, -90, -200, -1e30, 1e30])
+    x = torch.cat([g, torch.ones_like(g)], 1)
+    eye, no = torch.eye(64, device="cuda", dtype=torch.bfloat16), torch.zeros(64, 64, device="cuda", dtype=torch.bfloat16)
+    up = no.clone()
+    up[:, 0] = 1
+    got = gemm(2, x, torch.cat([eye, no], 1), torch.cat([no, up], 1))
+    want = g.double() / (1 + torch.exp(-g.double()))
+    want = torch.where(g < -88.7, 0.0, want)
+    assert bool(((got - want).abs() <= (2.0 ** -8 + 2.0 ** -20) * want.abs()).all())
+
+
 def test_fused_projection_rows_are_independent():
     """An infinity or NaN in a row of x stays in that row, the same bits with
     or without it; the same call twice gives the same bits."""
