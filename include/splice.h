@@ -120,6 +120,11 @@ typedef struct splice_desc splice_desc;
  *                 stored slots are the non-ZERO slots in slot order
  *                 (D_stored = splice_num_stored_donor_slots()).
  *
+ * A sequence's outputs do not depend, to the bit, on the order of the
+ * sequences or on any other sequence's L and W.  In a descriptor of other
+ * prompts, slots or numbers of sequences they agree within the rounding of
+ * the method's bf16 probabilities.
+ *
  * num_seqs >= 1, num_prompts >= 1, prompt_len >= 1, 1 <= num_donor_slots
  * <= 250, max_steps >= 1.  The clean and donor stores must each hold fewer
  * than 2^31 rows of d elements.  On success *out owns the descriptor; on

@@ -1052,10 +1052,12 @@ int prefix_tc_box_rows(int d) {
 }
 
 int prefix_tc_splits(int d, int p_vis, int max_splits, long spans, int sms, int* bounds) {
-    // Splits depend on the visible span length, the cap and the descriptor's
-    // prompts and donor slots (`spans`), never on the cells' L and W, so a
-    // row's arithmetic never depends on which other rows share its tile or on
-    // what they read.  Every item gathers its tile's queries and stores its
+    // Splits depend on the visible span length, the cap and, in a small launch
+    // (below), on how many tiles the descriptor's cells make of their prompts
+    // and donor slots (`spans`); never on the cells' L and W, so a row's
+    // arithmetic does not depend on which rows share its tile in a batch or on
+    // what they read.  In another batch it may, within the rounding of the
+    // probabilities, for a long span in a small launch.  Every item gathers its tile's queries and stores its
     // partial states, so long items move fewer bytes; but a launch ends as
     // unevenly as its last items are long.  So a span's first split is
     // kPrefixFirstSplitKeys keys and the rest kPrefixSplitKeys: the

@@ -4,7 +4,10 @@ on the CUDA path (no oracle involved):
 * C1 clean equivalence (§3): a cell that is never patched (L >= N or W > T)
   gives exactly the output of a clean-only batch;
 * C3 by reference == physical copy: reading donor spans through the
-  descriptor equals attention over a physically spliced per-sequence cache;
+  descriptor equals attention over a physically spliced per-sequence cache
+  (within the rounding of the probabilities, not bit for bit, for spans of
+  1024 keys or more in launches too small to fill the GPU, whose splits also
+  follow the number of tiles);
 * C5 W = 0 and W = 1 give the same run (reading of the onset);
 * C7 permuting the batch permutes the outputs;
 * the generated-span append writes exactly slot t - 1 (Algorithm 1).
@@ -85,34 +88,56 @@ def test_permutation_bit_exact():
             assert torch.equal(b.out, a.out[pc]), (l, t)
 
 
-def test_by_reference_equals_physical_copy():
-    wl = small_wl()
-    seqs = wl.sequences()
-    a = SweepBatch(wl, seqs=seqs)
-    Bn = len(seqs)
-    # one "prompt" per sequence holding the span it reads, every cell clean
+def physical_copy(a):
+    """The batch with every span copied: one "prompt" per sequence, which holds
+    the span that it reads (see load_spans), every cell clean."""
+    wl, Bn = a.wl, len(a.seqs)
     phys_wl = WL.Workload("phys", wl.num_layers, wl.num_q_heads, wl.num_kv_heads, wl.head_dim, Bn,
                           wl.prompt_len, (WL.BLANK,), wl.max_steps, (0,), (0,), 0, 0, batch=Bn)
-    phys_seqs = [WL.Seq(s, 0, wl.num_layers, 0) for s in range(Bn)]
-    b = SweepBatch(phys_wl, seqs=phys_seqs, fill=False)
+    b = SweepBatch(phys_wl, seqs=[WL.Seq(s, 0, wl.num_layers, 0) for s in range(Bn)], fill=False)
+    for store in (b.k_clean, b.v_clean, b.k_donor, b.v_donor):
+        store.zero_()
     b.k_suffix.copy_(a.k_suffix)
     b.v_suffix.copy_(a.v_suffix)
+    return b
+
+
+def load_spans(a, b, l, t):
+    """Copies what each sequence reads at (l, t); the source map."""
+    wl = a.wl
     stored = {k: i for i, k in enumerate(k for k, kd in enumerate(wl.slot_kinds) if kd != WL.ZERO)}
+    m = S.splice_debug_source_map(a.desc, l, t)
+    for s, q in enumerate(a.seqs):
+        p = q.prompt - a.p0
+        if m[s] == S.SRC_CLEAN:
+            b.k_clean[s, l].copy_(a.k_clean[p, l])
+            b.v_clean[s, l].copy_(a.v_clean[p, l])
+        elif m[s] == S.SRC_ZERO:
+            b.k_clean[s, l].zero_()
+            b.v_clean[s, l].zero_()
+        else:
+            st = stored[m[s] - S.SRC_DONOR0]
+            b.k_clean[s, l].copy_(a.k_donor[p, st, l])
+            b.v_clean[s, l].copy_(a.v_donor[p, st, l])
+    return m
+
+
+# Spans of less than 1024 keys, and longer ones in launches whose splits'
+# (tile, kv head) pairs are twice the multiprocessors or more, are split by
+# their length alone: the same bits.  (40 prompts and a donor each: 80 tiles of
+# 8 heads.)
+@pytest.mark.parametrize("Tp,P,cells", [(300, 2, None), (1500, 40, 160)])
+def test_by_reference_equals_physical_copy(Tp, P, cells):
+    wl = small_wl() if cells is None else WL.Workload(
+        "inv-long", 2, 16, 8, 64, P, Tp, (WL.SAME_ALGO, WL.ZERO), 12, (0, 2), (5,), 8, 4, batch=10 ** 6)
+    seqs = wl.sequences()
+    assert cells is None or len(seqs) == cells
+    a = SweepBatch(wl, seqs=seqs)
+    Bn = len(seqs)
+    b = physical_copy(a)
     for t in (1, 5, 12):
         for l in range(wl.num_layers):
-            m = S.splice_debug_source_map(a.desc, l, t)
-            for s, q in enumerate(seqs):
-                p = q.prompt - a.p0
-                if m[s] == S.SRC_CLEAN:
-                    b.k_clean[s, l].copy_(a.k_clean[p, l])
-                    b.v_clean[s, l].copy_(a.v_clean[p, l])
-                elif m[s] == S.SRC_ZERO:
-                    b.k_clean[s, l].zero_()
-                    b.v_clean[s, l].zero_()
-                else:
-                    st = stored[m[s] - S.SRC_DONOR0]
-                    b.k_clean[s, l].copy_(a.k_donor[p, st, l])
-                    b.v_clean[s, l].copy_(a.v_donor[p, st, l])
+            m = load_spans(a, b, l, t)
             a.gen_inputs(l, t)
             a.attn(l, t)
             b.q.copy_(a.q)
@@ -122,6 +147,61 @@ def test_by_reference_equals_physical_copy():
             assert torch.equal(a.out[nz], b.out[nz]), (l, t)
             if z:
                 assert_close(a.out[z].cpu().numpy(), b.out[z].cpu().numpy().astype(np.float64), f"zero l={l} t={t}")
+
+
+def split_bound(b, l, t, q):
+    """How far a row's output may move when its span is split elsewhere: a
+    probability is rounded to bf16 (within 2^-8 of it) relative to a maximum
+    that is the split's, once in either run, on top of fp32 sums; the sum of
+    |v| by weight is the attention over |V|."""
+    vc, vs = b.v_clean.clone(), b.v_suffix.clone()
+    b.v_clean.abs_()
+    b.v_suffix.abs_()
+    size = torch.empty_like(b.out)
+    b.attn(l, t, q=q, out=size)
+    b.v_clean.copy_(vc)
+    b.v_suffix.copy_(vs)
+    return (2 * 2.0 ** -8 * 1.01 + 2.0 ** -16) * size
+
+
+@pytest.mark.parametrize("Tp,d", [(1024, 128), (2500, 64), (4100, 256)])
+def test_a_long_span_in_a_small_launch_by_reference_and_by_copy(Tp, d):
+    """There the splits follow the number of tiles too (and so which cells share
+    a span): within the rounding of the probabilities."""
+    wl = WL.Workload("inv-small", 2, 4, 2, d, 1, Tp, (WL.SAME_ALGO, WL.BLANK), 12, (0, 1), (1, 5), 8, 4, batch=10 ** 6)
+    a = SweepBatch(wl, seqs=wl.sequences())
+    b = physical_copy(a)
+    for l, t in ((0, 1), (1, 5), (0, 12)):
+        load_spans(a, b, l, t)
+        a.gen_inputs(l, t)
+        a.attn(l, t)
+        b.attn(l, t, q=a.q)
+        assert bool(((a.out - b.out).abs() <= split_bound(b, l, t, a.q)).all()), (l, t)
+
+
+@pytest.mark.parametrize("Tp,d", [(300, 128), (2048, 128), (3000, 64), (4096, 256)])
+def test_a_cell_alone_and_in_a_large_batch(Tp, d):
+    """Its generated span is split by the batch's size, and a long prompt span
+    where a launch is small: within the rounding of the probabilities."""
+    wl = WL.Workload("inv-alone", 1, 8, 4, d, 30, Tp, (WL.SAME_ALGO,), 200, (0, 1), (1, 5), 8, 4, batch=10 ** 6)
+    seqs = wl.sequences()
+    a = SweepBatch(wl, seqs=seqs)
+    for s in (0, 1, len(seqs) - 1):
+        q = seqs[s]
+        one = SweepBatch(wl, seqs=[q], fill=False)
+        for name in ("k_clean", "v_clean", "k_donor", "v_donor"):
+            getattr(one, name).copy_(getattr(a, name)[q.prompt:q.prompt + 1])
+        one.k_suffix.copy_(a.k_suffix[s:s + 1])
+        one.v_suffix.copy_(a.v_suffix[s:s + 1])
+        for t in (3, 190):
+            a.gen_inputs(0, t)
+            a.attn(0, t)
+            one.attn(0, t, q=a.q[s:s + 1].contiguous())
+            vd = one.v_donor.clone()
+            one.v_donor.abs_()
+            bound = split_bound(one, 0, t, a.q[s:s + 1].contiguous())
+            one.v_donor.copy_(vd)
+            assert bool(((a.out[s:s + 1] - one.out).abs() <= bound).all()), (s, t)
 
 
 def test_append_writes_exactly_slot_t_minus_1():
