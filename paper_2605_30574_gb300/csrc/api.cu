@@ -547,7 +547,8 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
                                d->delta_on ? rows_d : rows_c};
         for (int i = 0; i < 6; ++i) {
             if (d->map_ptr[i] == mp[i]) continue;
-            if (splice::make_kv_tensor_map(d->maps[i], mp[i], mrows[i], sh.head_dim, box) != 0)
+            const int span_rows = i % 2 ? d->Tp : 0;    // V's by span
+            if (splice::make_kv_tensor_map(d->maps[i], mp[i], mrows[i], span_rows, sh.head_dim, box) != 0)
                 return fail(SPLICE_ECUDA, "cuTensorMapEncodeTiled failed for store %d", i);
             d->map_ptr[i] = mp[i];
         }

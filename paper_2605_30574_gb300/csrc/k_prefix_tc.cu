@@ -385,6 +385,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint64_t pol = tc::l2_policy_evict_first();
             uint64_t idle_since = 0;
             uint32_t spins = 0;
+            // V is loaded by span, so that a block that runs past the span's
+            // end holds zeros there: the next span's rows are none of this
+            // one's, and an infinity or NaN in them would get through a weight
+            // of 0.  (Of K's they make only logits that are dropped.  The
+            // number is divided out here, once per item: in the item's record
+            // it cost small launches of 256 dims 0.3 us.)
+            int v_span = 0;
             while (!(k_done && v_done)) {
                 bool prog = false;
                 if (!k_done) {
@@ -443,6 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         } else {
                             vi = inf;
                             vj = 0;
+                            v_span = int(unsigned(inf.span_row) / unsigned(P.Tp));
                             v_in = true;
                         }
                     }
@@ -451,12 +459,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const int stg = vg % C::VST;
                         if (tc::mbar_test_wait(bar(Bb::VEMPTY + stg), (uint32_t(vg / C::VST) & 1u) ^ 1u)) {
                             const CUtensorMap* tmv = vi.store == 0 ? &tm_vc : (vi.store == 1 ? &tm_vd : &tm_vx);
-                            const int y = int(vi.span_row + vi.k0 + vj * C::BN);
+                            const int y = vi.k0 + vj * C::BN;
                             tc::mbar_arrive_expect_tx(bar(Bb::VFULL + stg), C::KV_BYTES);
 #pragma unroll
                             for (int b = 0; b < C::KB; ++b)
-                                tc::tma_load_2d_hint(sbase + C::OFF_V + stg * C::KV_BYTES + b * (C::BN * 128), tmv, b * 64,
-                                                     y, bar(Bb::VFULL + stg), pol);
+                                tc::tma_load_3d_hint(sbase + C::OFF_V + stg * C::KV_BYTES + b * (C::BN * 128), tmv, b * 64,
+                                                     y, v_span, bar(Bb::VFULL + stg), pol);
                             ++vg;
                             ++vj;
                             prog = true;
@@ -1032,18 +1040,21 @@ constexpr double kBlockUs = 0.96, kBlockUs256 = 0.8, kItemUs = 2.2, kMergeUs = 2
 
 }  // namespace
 
-// 2D view [rows][d] of a bf16 store; box = 64 elements x box_rows rows, 128-byte swizzle.
-int make_kv_tensor_map(void* out_map, const void* base, long rows, int d, int box_rows) {
+// A bf16 store as [rows][d], or (span_rows > 0) as [spans][span_rows][d]; box =
+// 64 elements x box_rows rows, of one span, 128-byte swizzle, zeros outside.
+int make_kv_tensor_map(void* out_map, const void* base, long rows, int span_rows, int d, int box_rows) {
     EncodeFn enc = encode_fn();
     if (!enc) return int(cudaErrorNotSupported);
     if (rows < 1) rows = 1;
-    const cuuint64_t dims[2] = {cuuint64_t(d), cuuint64_t(rows)};
-    const cuuint64_t strides[1] = {cuuint64_t(d) * 2};
-    const cuuint32_t box[2] = {64, cuuint32_t(box_rows)};
-    const cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(static_cast<CUtensorMap*>(out_map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base),
-                     dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const bool by_span = span_rows > 0;
+    const cuuint64_t dims[3] = {cuuint64_t(d), cuuint64_t(by_span ? span_rows : rows),
+                                cuuint64_t(by_span ? std::max(rows / span_rows, 1L) : 1)};
+    const cuuint64_t strides[2] = {cuuint64_t(d) * 2, cuuint64_t(span_rows) * cuuint64_t(d) * 2};
+    const cuuint32_t box[3] = {64, cuuint32_t(box_rows), 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = enc(static_cast<CUtensorMap*>(out_map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, by_span ? 3 : 2,
+                     const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? 0 : int(cudaErrorInvalidValue);
 }
 

@@ -191,7 +191,7 @@ int launch_late_copy(void* dst, const void* src, size_t bytes, unsigned long lon
 int launch_wait_timeout(unsigned* err, unsigned long long limit_ns, void* stream);
 
 // Tensor-core prompt-span pass.  A tensor map is a 128-byte CUtensorMap.
-int make_kv_tensor_map(void* out_map, const void* base, long rows, int d, int box_rows);
+int make_kv_tensor_map(void* out_map, const void* base, long rows, int span_rows, int d, int box_rows);
 int prefix_tc_box_rows(int d);
 // Key splits of a visible span of p_vis keys in a launch of about `spans`
 // (tile, kv head) pairs on `sms` multiprocessors: returns their number n (at
@@ -201,7 +201,7 @@ int prefix_tc_box_rows(int d);
 int prefix_tc_splits(int d, int p_vis, int max_splits, long spans, int sms, int* bounds);
 // Estimated time of `items` items of up to `keys` keys on `ctas` CTAs, in us.
 double prefix_tc_us(int d, long items, int keys, int ctas);
-// maps: six tensor maps -- clean K, V; donor K, V; delta rows K, V.
+// maps: six tensor maps -- clean K, V; donor K, V; delta rows K, V; V's by span.
 // bounds: the span splits (p.nsp + 1 values); delta_keys: keys per split of
 // the delta rows.  overlap_previous: a programmatic dependent launch of the
 // preceding work on the stream.  With p.prefix_after_gs = 0 the kernel is

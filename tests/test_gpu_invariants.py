@@ -204,6 +204,37 @@ def test_a_cell_alone_and_in_a_large_batch(Tp, d):
             assert bool(((a.out[s:s + 1] - one.out).abs() <= bound).all()), (s, t)
 
 
+# spans that end inside a key block of 128 (64 of 256 dims), one that ends with
+# one; whole and through a window
+@pytest.mark.parametrize("Tp,window", [(1, 0), (70, 0), (128, 0), (300, 0), (300, 211), (1100, 0)])
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_a_row_does_not_see_the_spans_next_to_its_own(Tp, window, d):
+    """Infinities and NaNs everywhere but in the layer at hand change no bit;
+    in delta mode (whose splits follow the longest encoding of any layer) the
+    outputs stay finite and close."""
+    wl = WL.Workload("inv-next", 3, 8, 2, d, 2, Tp, (WL.SAME_ALGO, WL.ZERO, WL.BLANK), 12, (0, 2), (0, 5), 0, 0,
+                     batch=10 ** 6, sliding_window=window)
+    a = SweepBatch(wl, seqs=wl.sequences())
+    want = {(l, t): a.run(l, t).clone() for l, t in ((0, 12), (1, 5))}
+    stores = a.k_clean, a.v_clean, a.k_donor, a.v_donor
+    whole = [s.clone() for s in stores]
+    for (l, t), ref in want.items():
+        rest = [i for i in range(wl.num_layers) if i != l]
+        for s, value in zip(stores, (float("nan"), float("inf"), float("inf"), float("nan"))):
+            s[..., rest, :, :, :] = value
+        assert torch.equal(a.run(l, t), ref), (l, t)
+        if not window:
+            buf = torch.empty(S.splice_delta_bytes(a.desc), dtype=torch.uint8, device="cuda")
+            S.splice_delta_build(a.desc, *stores, buf)
+            out = a.run(l, t)
+            assert bool(out.isfinite().all())
+            assert_close(out.cpu().numpy(), ref.cpu().numpy().astype(np.float64), f"delta l={l} t={t}")
+            S.splice_delta_clear(a.desc)
+        for s, w in zip(stores, whole):
+            s.copy_(w)
+    S.splice_check_device_error(a.desc)
+
+
 def test_append_writes_exactly_slot_t_minus_1():
     wl = small_wl()
     a = SweepBatch(wl, seqs=wl.sequences())
