@@ -100,9 +100,11 @@ int launch_append(const uint16_t* kn, const uint16_t* vn, uint16_t* ks, uint16_t
 
 int launch_merge(const AttnParams& p, void* stream, bool overlap_previous) {
     const long rows = long(p.B) * p.Hq;
-    // the most partials a row can have: the prompt-span splits (none for a
-    // ZERO row), the generated-span splits and a delta row's splits
+    // the most partials a row can have (row_parts): the prompt-span splits
+    // (none for a ZERO row), the generated-span splits and a delta row's splits
     const int partials = p.nsp + p.nss + (p.delta_on ? p.nsd : 0);
+    static_assert(kMaxSplits <= 16, "the merge kernels take up to 16 partials");
+    if (partials > kMaxSplits) return int(cudaErrorInvalidValue);
     cudaLaunchConfig_t cfg = {};
     cfg.stream = static_cast<cudaStream_t>(stream);
     cudaLaunchAttribute attr[1];

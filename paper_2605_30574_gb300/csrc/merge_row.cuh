@@ -56,19 +56,18 @@ __device__ __forceinline__ float merge_weights(const AttnParams& P, int lane, in
     return den > 0.f ? 1.f / den : 0.f;
 }
 
-// Rows with at most NF partials (false, and nothing written, for another):
-// every load of the row -- lane i's
-// (m, l) of partial i and this lane's 16-byte slices of o of every partial --
-// is issued before any of them is used, so a row costs one round trip.
+// A row of at most NF partials (the caller's to see to: launch_merge): every load
+// of the row -- lane i's (m, l) of partial i and this lane's 16-byte slices of o
+// of every partial -- is issued before any of them is used, so a row costs one
+// round trip.
 template <int D, int NF>
-__device__ __forceinline__ bool merge_row_fast(const AttnParams& P, long row, int lane) {
+__device__ __forceinline__ void merge_row_fast(const AttnParams& P, long row, int lane) {
     constexpr int C4 = D / 4;                    // float4 slices of a row
     constexpr int SL = (C4 + 31) / 32;           // slices per lane
     const int s = int(row / P.Hq);
     const uint8_t code = P.src[s];
     const RowParts rp = row_parts(P, code);
     const int n = rp.span + rp.suffix + rp.delta;
-    if (n > NF) return false;
     const size_t plane = size_t(P.B) * P.Hq;
     float2 ml = make_float2(-INFINITY, 0.f);
     if (lane < n) ml = __ldcg(P.ws_ml + size_t(merge_slot(lane, rp)) * plane + row);
@@ -106,18 +105,16 @@ __device__ __forceinline__ bool merge_row_fast(const AttnParams& P, long row, in
         const int c = lane + 32 * q;
         if (c < C4) out[c] = make_float4(acc[q].x * inv, acc[q].y * inv, acc[q].z * inv, acc[q].w * inv);
     }
-    return true;
 }
 
 // RPW rows per warp (2 or 4), 32 / RPW lanes per row (lanes 0-15 row0,
-// 16-31 row0 + 1 for RPW = 2), for rows of at most NF live partials each:
-// the loads of all the warp's rows go out at once.  The reductions run over
-// the row's lanes with the partials on its first n lanes, so they add the
-// same values in the same order as merge_weights over 32 lanes (the other
-// lanes hold zeros): the same bits as merge_row_fast.  False (nothing
-// written) if any of the rows has more partials.
+// 16-31 row0 + 1 for RPW = 2), for rows of at most NF partials each: the loads
+// of all the warp's rows go out at once.  The reductions run over the row's
+// lanes with the partials on its first n lanes, so they add the same values in
+// the same order as merge_weights over 32 lanes (the other lanes hold zeros):
+// the same bits as merge_row_fast.
 template <int D, int NF, int RPW>
-__device__ __forceinline__ bool merge_rows_group(const AttnParams& P, long row0, int lane) {
+__device__ __forceinline__ void merge_rows_group(const AttnParams& P, long row0, int lane) {
     constexpr int LPR = 32 / RPW;                // lanes per row
     static_assert(NF <= LPR, "a row's partials sit on its first lanes");
     constexpr int C4 = D / 4;                    // float4 slices of a row
@@ -133,7 +130,6 @@ __device__ __forceinline__ bool merge_rows_group(const AttnParams& P, long row0,
         rp = row_parts(P, code);
     }
     const int n = rp.span + rp.suffix + rp.delta;
-    if (!__all_sync(0xffffffffu, n <= NF)) return false;
     const size_t plane = size_t(total);
     float2 ml = make_float2(-INFINITY, 0.f);
     if (hl < n) ml = __ldcg(P.ws_ml + size_t(merge_slot(hl, rp)) * plane + row);
@@ -183,7 +179,6 @@ __device__ __forceinline__ bool merge_rows_group(const AttnParams& P, long row0,
             if (c < C4) out[c] = make_float4(acc[q].x * inv, acc[q].y * inv, acc[q].z * inv, acc[q].w * inv);
         }
     }
-    return true;
 }
 
 }  // namespace splice

@@ -388,6 +388,67 @@ def test_causal_attention_is_the_same_every_time(hq, hkv, d):
     K.check_device_error()
 
 
+# one tile per pair of CTAs and shares of K; tiles by waves, with a tail; the
+# library's head (more than 256 rows)
+@pytest.mark.parametrize("rows", [9, 300])
+def test_a_captured_graph_of_the_pieces(rows):
+    """Replayed on other inputs in the same buffers: the eager calls' bits."""
+    model = RandomDecoder(DecoderDims(1, 6, 2, 128, 1024, 9000, 500), seed=4)
+    g = gen(rows)
+    h, attn, pos = randn(g, rows, 1024), randn(g, rows, 6, 128), torch.arange(rows, device="cuda")
+    tokens = torch.randint(0, 500, (rows,), generator=g, device="cuda")
+    k, v = (torch.zeros(1, 2, rows, 128, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+
+    def pieces():
+        return (*model.qkv(0, h, pos), model.block_out(0, h, attn), model.logits(h), model.prefill(tokens, k, v), k, v)
+
+    with torch.no_grad():
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            pieces()
+        torch.cuda.current_stream().wait_stream(side)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            out = pieces()
+        for _ in range(3):
+            for x, new in ((h, randn(g, rows, 1024)), (attn, randn(g, rows, 6, 128)), (pos, pos + 77),
+                           (tokens, tokens.flip(0).clone())):
+                x.copy_(new)
+            want = [t.clone() for t in pieces()]
+            for t in out:
+                t.fill_(float("nan"))
+            graph.replay()
+            assert all(torch.equal(a, b) for a, b in zip(out, want))
+    K.check_device_error()
+
+
+def test_two_streams_at_once():
+    """Layers on two streams, each in its own order, with the scratch and the
+    outputs of many calls in flight: the bits of each alone."""
+    models = [RandomDecoder(DecoderDims(1, 8, 2, 128, 2048, 5000, 700), seed=i) for i in range(2)]
+    g = gen(6)
+    work = [[(randn(g, n, 2048), randn(g, n, 8, 128), torch.arange(n, device="cuda")) for n in rows]
+            for rows in ((1, 40, 300, 700), (513, 7, 130, 256))]
+
+    def pieces(m, h, attn, pos):
+        q, k, v = m.qkv(0, h, pos)
+        return (q, k, v, m.block_out(0, h, attn), m.logits(h),
+                K.causal(q, k.transpose(0, 1).contiguous(), v.transpose(0, 1).contiguous(), 0.1))
+
+    want = [[pieces(m, *w) for w in ws] for m, ws in zip(models, work)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    got = []
+    for i in range(40):
+        for m, ws, wants, stream in zip(models, work, want, streams):
+            with torch.cuda.stream(stream):
+                got.append((pieces(m, *ws[i % 4]), wants[i % 4]))
+    K.check_device_error()
+    for a, b in got:
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
 @pytest.mark.skipif(torch.cuda.device_count() < 2, reason="one device")
 def test_a_second_device():
     """Both devices of a process, one after the other."""
