@@ -270,17 +270,18 @@ class RandomDecoder:
             if q.dtype is kh.dtype is vh.dtype is torch.bfloat16 and K.plain((q,), ()):
                 a = K.causal(q, kh.contiguous(), vh.contiguous(), self.sm_scale)
                 if a is not None:
-                    h = self.block_out(l, h, a)
+                    h = self.block_out(l, h, a if _own(self, "block_out") else a.float())
                     continue
             kh, vh = kh[None], vh[None]
             qh = q.transpose(0, 1)[None]                    # [1, Hq, T_p, d]
             a = torch.nn.functional.scaled_dot_product_attention(qh, kh, vh, is_causal=True, scale=self.sm_scale,
                                                                  enable_gqa=G > 1)
-            h = self.block_out(l, h, a[0].transpose(0, 1).contiguous())
+            a = a[0].transpose(0, 1)
+            h = self.block_out(l, h, a.contiguous() if _own(self, "block_out") else a.float())
         return self.logits(h[-1])
 
 
-_PIECES = {name: getattr(RandomDecoder, name) for name in ("rope", "qkv")}
+_PIECES = {name: getattr(RandomDecoder, name) for name in ("rope", "qkv", "block_out")}
 
 
 def _own(model: RandomDecoder, name: str) -> bool:

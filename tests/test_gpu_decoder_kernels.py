@@ -181,6 +181,20 @@ def test_prefill_into_stores_and_into_copies(hq, hkv, d, T):
     assert torch.equal(k.float(), kf) and torch.equal(v.float(), vf) and torch.equal(got, want)
 
 
+def test_prefill_gives_a_block_out_of_ones_own_fp32():
+    dims, kinds = DecoderDims(2, 4, 2, 64, 128, 64, 50), []
+
+    class Own(RandomDecoder):
+        def block_out(self, l, h, attn):
+            kinds.append(attn.dtype)
+            return super().block_out(l, h, attn)
+
+    tokens = torch.arange(9, device="cuda")
+    stores = [torch.zeros(2, 2, 9, 64, device="cuda", dtype=torch.bfloat16) for _ in range(2)]
+    assert torch.equal(Own(dims).prefill(tokens, *stores), RandomDecoder(dims).prefill(tokens, *stores))
+    assert kinds == [torch.float32] * 2
+
+
 def test_prefill_writes_its_stores_as_torch_does():
     """A graph that saved a store sees that it was written since; a store of
     inference mode is refused outside it."""

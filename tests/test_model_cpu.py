@@ -141,3 +141,18 @@ def test_a_piece_of_ones_own_is_the_one_that_runs(monkeypatch):
     assert not _own(b, "qkv")
     monkeypatch.setattr(RandomDecoder, "rope", Unturned.rope)
     assert not plain._kernels(0, h, pos)
+
+
+class Scaled(RandomDecoder):
+    """Its own block_out, which reads the attention output as fp32."""
+
+    def block_out(self, l, h, attn):
+        assert attn.dtype is torch.float32
+        return super().block_out(l, h, attn * torch.ones((), dtype=torch.float32))
+
+
+def test_a_block_out_of_ones_own_gets_the_attention_in_fp32():
+    dims = DecoderDims(1, 2, 1, 64, 64, 64, 8)
+    stores = [torch.zeros(1, 1, 5, 64, dtype=torch.bfloat16) for _ in range(2)]
+    got = Scaled(dims, device="cpu").prefill(torch.arange(5), *stores)
+    assert torch.equal(got, RandomDecoder(dims, device="cpu").prefill(torch.arange(5), *stores))
