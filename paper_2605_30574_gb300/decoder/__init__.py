@@ -206,17 +206,20 @@ def causal(q, k, v, scale):
     """Causal attention of q [T, Hq, d] over k, v [Hkv, T, d], bf16 and
     contiguous: [T, Hq, d] bf16; None for the shapes it does not take."""
     T, hq, d = q.shape
-    if T > 1 << 20 or d not in (64, 128, 256) or not _aligned(q, k, v):
+    hkv = k.shape[0]
+    if T > 1 << 20 or d not in (64, 128, 256) or hq % hkv or not k.shape == v.shape == (hkv, T, d) or not _aligned(q, k, v):
         return None
     out = torch.empty_like(q)
-    _launch("decoder_causal", q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), T, hq, k.shape[0], d, scale)
+    _launch("decoder_causal", q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), T, hq, hkv, d, scale)
     return out
 
 
 # Up to this many rows the fused projections stream a large weight matrix faster
 # than the library (151936 x 4096, fp32 out: 1 row 178 us against 205, 256 rows
 # 224 against 237); with more, and two tiles of rows, they do not (320 rows 271
-# against 257, 400 rows 320 against 298).
+# against 257, 400 rows 320 against 298; of 151936 x 1024 108 against 97).  A
+# small matrix is a question of host time, which the line does not look at: 4096
+# x 1024 takes 27 us against 73 at any number of rows.
 LOGITS_ROWS = 256
 
 

@@ -267,8 +267,9 @@ class RandomDecoder:
                 kl.copy_(k.transpose(0, 1))
                 vl.copy_(v.transpose(0, 1))
                 kh, vh = k.transpose(0, 1), v.transpose(0, 1)
-            if q.dtype is kh.dtype is vh.dtype is torch.bfloat16 and K.plain((q,), ()):
-                a = K.causal(q, kh.contiguous(), vh.contiguous(), self.sm_scale)
+            if q.dtype is kh.dtype is vh.dtype is torch.bfloat16:
+                kc, vc = kh.contiguous(), vh.contiguous()
+                a = K.causal(q, kc, vc, self.sm_scale) if K.plain((q, kc, vc), ()) else None
                 if a is not None:
                     h = self.block_out(l, h, a if _own(self, "block_out") else a.float())
                     continue

@@ -156,3 +156,13 @@ def test_a_block_out_of_ones_own_gets_the_attention_in_fp32():
     stores = [torch.zeros(1, 1, 5, 64, dtype=torch.bfloat16) for _ in range(2)]
     got = Scaled(dims, device="cpu").prefill(torch.arange(5), *stores)
     assert torch.equal(got, RandomDecoder(dims, device="cpu").prefill(torch.arange(5), *stores))
+
+
+# (other lengths, head dims and head counts than the queries'; unlike shapes)
+@pytest.mark.parametrize("k,v", [((2, 5, 64), (2, 5, 64)), ((2, 7, 64), (2, 7, 64)), ((2, 6, 128), (2, 6, 128)),
+                                 ((3, 6, 64), (3, 6, 64)), ((2, 6, 64), (2, 5, 64)), ((2, 6, 64), (1, 6, 64)),
+                                 ((2, 6, 64), (2, 6, 128))])
+def test_prefill_attention_kernel_takes_matching_keys_only(k, v):
+    """A qkv of one's own may return others, which torch's attention refuses."""
+    q, k, v = (torch.zeros(s, dtype=torch.bfloat16) for s in ((6, 4, 64), k, v))
+    assert K.causal(q, k, v, 0.125) is None
