@@ -59,8 +59,8 @@ NOMINAL_HBM_GBS = 8000.0
 # reduced ladder case (read + written bytes / algorithmic bytes of that launch);
 # traffic grows in proportion to the units a launch processes.  Only kernels
 # whose current build was captured are listed.
-TRAFFIC_PER_ALGORITHMIC_BYTE = {"generated_span_pass": (539.047 + 6.002) / 541.065,
-                                "prompt_span_pass": (236.984 + 4.786) / 234.881}
+TRAFFIC_PER_ALGORITHMIC_BYTE = {"generated_span_pass": (539.078 + 5.797) / 541.065,
+                                "prompt_span_pass": (236.993 + 4.759) / 234.881}
 
 
 def step_schedule(T: int, n: int, offset: int = 0):

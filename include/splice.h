@@ -279,7 +279,9 @@ splice_status spliced_decode_attn_static(splice_desc* desc, int layer, int step,
  * of attention over the clean span without those positions and attention
  * over the encoded rows.  In delta mode the readers of an encoded slot are
  * stacked into the clean span's tiles (their encoded positions dropped row
- * by row) and read the encoded rows as tiles of their own.
+ * by row) and read the encoded rows as tiles of their own.  (A dropped
+ * position has weight 0, which an infinity or NaN in the clean span's V row
+ * there gets through.)
  *
  * splice_delta_bytes -- bytes of the delta buffer of this descriptor (0 for
  * NULL or when no slot is stored).  Layout, each part starting on a 256-byte

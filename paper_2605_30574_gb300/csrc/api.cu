@@ -490,11 +490,14 @@ splice_status attn_common(splice_desc* d, int layer, int step, const splice_bf16
     // from half of them, while the prompt-span pass, a chain of latencies, uses
     // little of it.  As few CTAs as end within kPrefixShare of the
     // generated-span pass's time (and before its warps have more items to
-    // merge later than they keep).  Measured at 152, 96, 76 and 56 CTAs: eight
-    // rows per kv head, 300 cells, 79.7, 75.4, 74.9, 74.7 us; Qwen3-4B-shaped
-    // 118.0, 116.4, 115.7, 115.1; where the prompt spans hold more, it costs
-    // (252 cells of 2255 keys: 69.8, 102.1), and where the generated-span pass
-    // is short of warps itself (seven rows of 256 dims: 141.7, 141.9, 149).
+    // merge later than they keep), of 6/19 to 16/19 of the SMs.  Measured at all
+    // 152 and at the counts tried, 128, 112, 96, 80, 64, 48: eight rows per kv
+    // head, 300 cells, prompts of 777 keys, 80.6, 78.8, 77.3, 76.8, 74.9, 75.0,
+    // 74.3 us; Qwen3-4B-shaped 118.5, 118.3, 117.3, 116.9, 116.5, 116.2, 116.3;
+    // where the prompt spans hold too much for the rule, few CTAs cost (252
+    // cells, sixteen rows, prompts of 2255 keys: 104.8, ..., 101.0, 114.4), and
+    // so they do where the generated-span pass is short of warps itself (seven
+    // rows of 256 dims: 63.8, ..., 64.3, 65.9).
     if (p.gs_after_prefix && splice::generated_span_streams_from_half(sh.head_dim, p.gs_rows)) {
         const double gs_us = double(gs_keys) * sh.head_dim * 4 / kGenBytesPerUs;
         const double per_warp = double(d->B) * sh.num_kv_heads * p.gs_chunks * p.nss /

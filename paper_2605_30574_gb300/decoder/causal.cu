@@ -13,7 +13,7 @@
 // kv head next to one another.  O is rescaled where a row's maximum grows, so
 // that the largest weight is 1 exactly (left up to 2^8 behind, 7% faster but 3%
 // further from 64 bits).  32 heads of 128, 8 for keys, against the flash kernel
-// that torch picks: 256 tokens 7.6 us, 16.2; 1024 22.1, 53.4; 4096 142, 427; no
+// that torch picks: 256 tokens 7.2 us, 16.2; 1024 22.9, 53.4; 4096 143, 427; no
 // further from 64 bits at any size.
 //
 // Every wait is bounded, as in gemm.cu.

@@ -15,7 +15,7 @@
 // that are bound by their loads' latency, not by bandwidth.  Their point is
 // their number: in a Qwen3-8B-shaped layer of 512 cells they take the place
 // of 62 launches by 7 (980 -> 317 us with library GEMMs; a step of two layers and
-// the head 2149 -> 797, a prefill of 1024 tokens 2376 -> 890; 216, 700 and 774
+// the head 2149 -> 797, a prefill of 1024 tokens 2376 -> 890; 216, 705 and 773
 // with gemm.cu and causal.cu).  Times below are a launch's
 // on cold caches at 512 rows of 4096 (32 + 2 x 8 heads of 128, F = 12288).
 #include <cuda_bf16.h>

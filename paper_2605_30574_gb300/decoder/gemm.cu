@@ -33,7 +33,7 @@
 // keys): 768 rows 855 -> 545 us, 1024 858 -> 682, 1536 970 -> 965, 4096 2870 ->
 // 2767; d_model 5120, F 17408: 1024 1054 -> 1066, 4096 4356 -> 4227 (all before
 // the smaller tiles of the last wave, see plan).  A decoder layer of 512 cells
-// took 317 so, 248 with one CTA to a tile, 215 now.
+// took 317 so, 248 with one CTA to a tile, 216 now.
 //
 // Every wait is bounded; one that runs out sets the error word, and every role
 // leaves its loop (see decoder_error).
