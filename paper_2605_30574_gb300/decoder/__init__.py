@@ -55,12 +55,14 @@ def lib() -> ctypes.CDLL:
 def plain(acts, weights) -> bool:
     """Whether the kernels may stand in for the torch expressions on these
     activations and bf16 weights."""
+    if torch.compiler.is_compiling():       # (first: a compiler cannot trace the rest)
+        return False
     dev = acts[0].device
     if dev.type != "cuda" or dev.index != torch.cuda.current_device():
         return False
     if (torch._C._are_functorch_transforms_active() or torch._C._len_torch_dispatch_stack()
             or torch._C._len_torch_function_stack() or torch.is_autocast_enabled() or _fwad._current_level >= 0
-            or torch.compiler.is_compiling() or torch.jit.is_tracing()):
+            or torch.jit.is_tracing()):
         return False
     grad = torch.is_grad_enabled()
     for t in acts:

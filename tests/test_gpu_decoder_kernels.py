@@ -149,6 +149,25 @@ def test_transforms_modes_and_other_types_take_the_torch_path():
     assert tangent.abs().max() > 0
 
 
+def test_compilers_and_tracers_see_the_torch_expressions():
+    """A whole graph without a break, a trace and a proxy's graph, each of
+    which runs other inputs as the torch expressions do (bit for bit)."""
+    from torch.fx.experimental.proxy_tensor import make_fx
+    model = RandomDecoder(DecoderDims(1, 4, 2, 64, 128, 64, 50), seed=0)
+    h, other, attn, pos = randn(gen(), 6, 128), randn(gen(1), 6, 128), randn(gen(2), 6, 4, 64), torch.arange(6, device="cuda")
+    pieces = (lambda x: model.qkv(0, x, pos)[0], lambda x: model.block_out(0, x, attn), lambda x: model.logits(x))
+    k, v = (torch.zeros(1, 2, 6, 64, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    for f in pieces:
+        want = f(other.clone().requires_grad_()).detach()
+        with torch.no_grad():
+            torch._dynamo.reset()
+            for g in (torch.compile(f, backend="eager", fullgraph=True), torch.jit.trace(f, (h,), check_trace=False),
+                      make_fx(f)(h)):
+                assert torch.equal(g(other), want)
+    torch._dynamo.reset()
+    assert model.prefill(pos, k, v).isfinite().all()
+
+
 def test_tensors_whose_values_are_not_at_their_address_take_the_torch_path():
     model = RandomDecoder(DecoderDims(1, 4, 2, 64, 128, 64, 50), seed=0)
     h, pos = randn(gen(), 6, 128), torch.arange(6, device="cuda")
